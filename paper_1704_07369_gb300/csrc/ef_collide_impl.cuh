@@ -76,6 +76,17 @@ struct Sync {
             asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         }
     }
+    // war() in two halves, for work between them that neither reads nor writes what the barrier
+    // protects; every thread calls both, in turn (a one-CTA cluster waits in the second)
+    __device__ __forceinline__ void war_arrive()
+    {
+        if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    }
+    __device__ __forceinline__ void war_wait()
+    {
+        if (C == 1) __syncthreads();
+        else asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    }
 };
 
 __device__ __forceinline__ void record_status(int *status, int code)

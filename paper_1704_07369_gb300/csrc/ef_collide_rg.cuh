@@ -95,7 +95,7 @@ template <int N>
 __host__ __device__ constexpr size_t rg_smem_bytes(int planes, int npc, bool g_shared)
 {
     return (size_t)2 * planes * rg_plane_stride<N>() * 8 + (size_t)N * npc * 8 + (g_shared ? (size_t)planes * N * N * 4 : 0) +
-           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float);
+           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float) + N * sizeof(uint32_t);
 }
 
 // lanes of the calling thread's warp that exist: a block whose size is not a multiple of 32 has a
@@ -111,36 +111,32 @@ template <int N>
 __device__ __forceinline__ int rg_poff(int q) { return rg_at<N>(q / (N / 2), q % (N / 2)); }
 
 // stage-A scatter of one pencil (lane pairs hold pencils q, q + 1 of one slab row; one shuffle per
-// z pair so that each lane issues 16-byte stores; owner CTA of z by multiply-high)
+// z pair so that each lane issues 16-byte stores).  zt[z] is the shared::cluster address of plane z in
+// its owner's first slab (a table in shared memory: one broadcast load in place of the owner's
+// division and mapa), off the byte offset of the slab and the pencil pair.
 template <int N>
-__device__ __forceinline__ void rg_scatter(const C2<float> (&v)[N], uint32_t slab_base, int P, unsigned long long pm,
-                                           int poff, bool odd, unsigned mask)
+__device__ __forceinline__ void rg_scatter(const C2<float> (&v)[N], const uint32_t *zt, uint32_t off, bool odd, unsigned mask)
 {
-    constexpr int NPP = rg_plane_stride<N>();
+    const uint32_t *zo = zt + (odd ? 1 : 0);
 #pragma unroll
     for (int z0 = 0; z0 < N; z0 += 2) {
         const C2<float> send = odd ? v[z0] : v[z0 + 1];
         C2<float> recv;
         recv.x = __shfl_xor_sync(mask, send.x, 1);
         recv.y = __shfl_xor_sync(mask, send.y, 1);
-        const int z = odd ? z0 + 1 : z0;
         const C2<float> lo = odd ? recv : v[z0];
         const C2<float> hi = odd ? v[z0 + 1] : recv;
-        const int owner = plane_owner(z, pm), zl = z - owner * P;
-        st_cluster(cluster_map(slab_base + (uint32_t)((zl * NPP + poff) * 8), owner), make_float4(lo.x, lo.y, hi.x, hi.y));
+        st_cluster(zo[z0] + off, make_float4(lo.x, lo.y, hi.x, hi.y));
     }
 }
 
 template <int N>
-__device__ __forceinline__ void rg_gather(C2<float> (&v)[N], uint32_t slab_base, int P, unsigned long long pm, int poff,
-                                          bool odd, unsigned mask)
+__device__ __forceinline__ void rg_gather(C2<float> (&v)[N], const uint32_t *zt, uint32_t off, bool odd, unsigned mask)
 {
-    constexpr int NPP = rg_plane_stride<N>();
+    const uint32_t *zo = zt + (odd ? 1 : 0);
 #pragma unroll
     for (int z0 = 0; z0 < N; z0 += 2) {
-        const int z = odd ? z0 + 1 : z0;
-        const int owner = plane_owner(z, pm), zl = z - owner * P;
-        const float4 w = ld_cluster_f4(cluster_map(slab_base + (uint32_t)((zl * NPP + poff) * 8), owner));
+        const float4 w = ld_cluster_f4(zo[z0] + off);
         const C2<float> lo = C2<float>{w.x, w.y}, hi = C2<float>{w.z, w.w};
         const C2<float> send = odd ? lo : hi;
         C2<float> recv;
@@ -299,9 +295,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
     long long *s_cell = reinterpret_cast<long long *>(part + (32 + 1) * kDiag);
     int *s_nubig = reinterpret_cast<int *>(s_cell + 1);
     float *s_maxnu = reinterpret_cast<float *>(s_cell + 2);          // [32 warps] max nu of the loss op
-    const uint32_t base0 = smem_u32addr(Is0), base1 = smem_u32addr(Is1);
+    uint32_t *s_zt = reinterpret_cast<uint32_t *>(s_maxnu + 32);     // [N] cluster addresses of the planes
+    const uint32_t base0 = smem_u32addr(Is0), slab1 = (uint32_t)((size_t)P * NPP * sizeof(C2<T>));
+    for (int z = tid; z < N; z += nt) s_zt[z] = cluster_map(base0 + (uint32_t)((z % P) * NPP * sizeof(C2<T>)), z / P);
 
-    const unsigned long long pm = (0x100000000ull + (unsigned)P - 1u) / (unsigned)P;
     const int64_t nclusters = gridDim.x / C;
     const int64_t cid = blockIdx.x / C;
     const int lane = tid & 31;
@@ -365,7 +362,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             if (has) {
                 const int q = rank * NPC + ql;
                 C2<T> v[N];
-                rg_gather<N>(v, base0, P, pm, rg_poff<N>(q & ~1), q & 1, mask);
+                rg_gather<N>(v, s_zt, (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
                 fft<N, -1, N>(v);
 #pragma unroll
                 for (int z = 0; z < N; ++z) Fs[(size_t)z * NPC + ql] = cscale(v[z], scale);
@@ -384,21 +381,31 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             // ---------------- A: multiply, axis 0 inverse, scatter (one (direction, pencil) item
             // per thread; lanes of a pair share the direction since NPC is even)
             const int nitems = (pair ? 2 : 1) * NPC;
+            bool held = o > 0;             // the previous op's slabs are not yet known to be read by all
             for (int q0 = tid - lane; q0 < nitems; q0 += nt) {
                 const int qi = q0 + lane;
                 const bool has = qi < nitems;
                 const unsigned mask = __ballot_sync(wmask, has);
-                if (has) {
-                    const int b = qi >= NPC;
-                    const int ql = qi - b * NPC;
-                    const int q = rank * NPC + ql;
-                    const int ky = q / NH, kx = q % NH;
-                    const T *M = Mbase + (size_t)(b ? op.dir2 : op.dir) * N * NPT + ky * H + kx;
-                    C2<T> v[N];
+                const int qc = has ? qi : nitems - 1;      // lanes past the end repeat the last item, unstored
+                const int b = qc >= NPC;
+                const int ql = qc - b * NPC;
+                const int q = rank * NPC + ql;
+                const int ky = q / NH, kx = q % NH;
+                const T *M = Mbase + (size_t)(b ? op.dir2 : op.dir) * N * NPT + ky * H + kx;
+                C2<T> v[N];
 #pragma unroll
-                    for (int z = 0; z < N; ++z) v[z] = cscale(Fs[(size_t)z * NPC + ql], __ldg(M + (size_t)z * NPT));
-                    fft<N, 1, N>(v);
-                    rg_scatter<N>(v, b ? base1 : base0, P, pm, rg_poff<N>(q & ~1), q & 1, mask);
+                for (int z = 0; z < N; ++z) v[z] = cscale(Fs[(size_t)z * NPC + ql], __ldg(M + (size_t)z * NPT));
+                fft<N, 1, N>(v);
+                // the transform above touches nothing that the other CTAs still read: only the scatter
+                // waits for their arrival at the end of the previous op (with the plane address table:
+                // 2048 cells of N = 32 2.329 -> 2.288 ms, 256 of N = 64 5.32 -> 5.24 ms)
+                if (held) {
+                    __syncwarp(wmask);
+                    bar.war_wait();
+                    held = false;
+                }
+                if (has) {
+                    rg_scatter<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
                     if (a.prefetch && o + 1 < a.nops) {
                         // pull the next op's multipliers of this item towards L1 while the local
                         // passes run (the next op has the same item split: both directions or, after
@@ -410,6 +417,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                     }
                 }
             }
+            if (held) bar.war_wait();      // warps without an item
             bar.full();
 
             // ---------------- B: axis 1 inverse on the stored k_x < N/2 columns of each slab
@@ -543,7 +551,9 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                 }
                 if (lane == 0) s_maxnu[tid >> 5] = mxt;
             }
-            bar.war();
+            // write-after-read: the next op's scatter waits for this arrival
+            bar.war_arrive();
+            if (o + 1 == a.nops) bar.war_wait();
         }
 
         // ---------------- per-cell reduction of the diagnostics
