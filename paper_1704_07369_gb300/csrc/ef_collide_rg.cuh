@@ -95,7 +95,7 @@ template <int N>
 __host__ __device__ constexpr size_t rg_smem_bytes(int planes, int npc, bool g_shared)
 {
     return (size_t)2 * planes * rg_plane_stride<N>() * 8 + (size_t)N * npc * 8 + (g_shared ? (size_t)planes * N * N * 4 : 0) +
-           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float) + N * sizeof(uint32_t);
+           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float) + N * sizeof(uint2) + 8;
 }
 
 // lanes of the calling thread's warp that exist: a block whose size is not a multiple of 32 has a
@@ -110,14 +110,61 @@ __device__ __forceinline__ unsigned warp_lanes(int nt, int tid)
 template <int N>
 __device__ __forceinline__ int rg_poff(int q) { return rg_at<N>(q / (N / 2), q % (N / 2)); }
 
+// Clusters of at least this many CTAs scatter by st.async: every store counts its bytes on the receiving
+// CTA's mbarrier, and a CTA waits for its own slabs to be full in place of the release / acquire cluster
+// barrier, whose membar waits for the sender's remote stores to be acknowledged (membar and barrier
+// stalls were a quarter of the N = 48 kernel's, and the CTAs of a large cluster drift apart).  4096
+// ragged cells (clusters of 12 and 10) 11.64 -> 10.33 ms, 256 cells of N = 64 (16) 5.34 -> 4.59 ms, 512
+// of N = 32 on clusters of 4 0.643 -> 0.617 ms; clusters of 1 and 2 keep the barrier (N = 24 on one CTA
+// lost 19%, N = 32 on two 5%: the byte counts of mostly local stores cost more than the barrier).  A
+// template parameter: one kernel with both scatters lost 1.5 - 2.5% to its size.
+constexpr int kRgAsync = 3;
+
+__device__ __forceinline__ void st_async(uint32_t a, C2<float> v, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v.x),
+                 "f"(v.y), "r"(bar)
+                 : "memory");
+}
+
+// Wait for one phase of the CTA's slab mbarrier; gives up after about a second of device time (false).
+__device__ __forceinline__ bool slab_wait(uint32_t bar, uint32_t parity)
+{
+    uint64_t t0 = 0;
+    for (int it = 0;; ++it) {
+        uint32_t done;
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+        if ((it & 63) == 63) {
+            uint64_t t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > 1000000000ull) return false;
+        }
+    }
+}
+
+// the whole pencil, one 8-byte store per plane (zt: plane address and its owner's mbarrier).  8-byte
+// stores without the shuffles were 1 - 2% faster here than 16-byte ones with them.
+template <int N>
+__device__ __forceinline__ void rg_scatter_async(const C2<float> (&v)[N], const uint2 *zt, uint32_t off)
+{
+#pragma unroll
+    for (int z = 0; z < N; ++z) {
+        const uint2 d = zt[z];
+        st_async(d.x + off, v[z], d.y);
+    }
+}
+
 // stage-A scatter of one pencil (lane pairs hold pencils q, q + 1 of one slab row; one shuffle per
-// z pair so that each lane issues 16-byte stores).  zt[z] is the shared::cluster address of plane z in
+// z pair so that each lane issues 16-byte stores).  zt[z].x is the shared::cluster address of plane z in
 // its owner's first slab (a table in shared memory: one broadcast load in place of the owner's
 // division and mapa), off the byte offset of the slab and the pencil pair.
 template <int N>
-__device__ __forceinline__ void rg_scatter(const C2<float> (&v)[N], const uint32_t *zt, uint32_t off, bool odd, unsigned mask)
+__device__ __forceinline__ void rg_scatter(const C2<float> (&v)[N], const uint2 *zt, uint32_t off, bool odd, unsigned mask)
 {
-    const uint32_t *zo = zt + (odd ? 1 : 0);
+    const uint2 *zo = zt + (odd ? 1 : 0);
 #pragma unroll
     for (int z0 = 0; z0 < N; z0 += 2) {
         const C2<float> send = odd ? v[z0] : v[z0 + 1];
@@ -126,17 +173,17 @@ __device__ __forceinline__ void rg_scatter(const C2<float> (&v)[N], const uint32
         recv.y = __shfl_xor_sync(mask, send.y, 1);
         const C2<float> lo = odd ? recv : v[z0];
         const C2<float> hi = odd ? v[z0 + 1] : recv;
-        st_cluster(zo[z0] + off, make_float4(lo.x, lo.y, hi.x, hi.y));
+        st_cluster(zo[z0].x + off, make_float4(lo.x, lo.y, hi.x, hi.y));
     }
 }
 
 template <int N>
-__device__ __forceinline__ void rg_gather(C2<float> (&v)[N], const uint32_t *zt, uint32_t off, bool odd, unsigned mask)
+__device__ __forceinline__ void rg_gather(C2<float> (&v)[N], const uint2 *zt, uint32_t off, bool odd, unsigned mask)
 {
-    const uint32_t *zo = zt + (odd ? 1 : 0);
+    const uint2 *zo = zt + (odd ? 1 : 0);
 #pragma unroll
     for (int z0 = 0; z0 < N; z0 += 2) {
-        const float4 w = ld_cluster_f4(zo[z0] + off);
+        const float4 w = ld_cluster_f4(zo[z0].x + off);
         const C2<float> lo = C2<float>{w.x, w.y}, hi = C2<float>{w.z, w.w};
         const C2<float> send = odd ? lo : hi;
         C2<float> recv;
@@ -262,7 +309,7 @@ __device__ __forceinline__ void diag_reduce_cell(const CollideArgs &a, const Dia
 
 // GS = false: G of this thread's RPT rows in registers (nt * RPT = rows); GS = true: G in shared
 // memory, column-major ([x][row], so consecutive threads touch consecutive banks), rows looped.
-template <int D, int N, int RPT, int LB, bool GS>
+template <int D, int N, int RPT, int LB, bool GS, bool ASYNC>
 __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
 {
     static_assert(D == 3, "3D only");
@@ -295,9 +342,17 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
     long long *s_cell = reinterpret_cast<long long *>(part + (32 + 1) * kDiag);
     int *s_nubig = reinterpret_cast<int *>(s_cell + 1);
     float *s_maxnu = reinterpret_cast<float *>(s_cell + 2);          // [32 warps] max nu of the loss op
-    uint32_t *s_zt = reinterpret_cast<uint32_t *>(s_maxnu + 32);     // [N] cluster addresses of the planes
+    uint2 *s_zt = reinterpret_cast<uint2 *>(s_maxnu + 32);           // [N] cluster address of a plane and its owner's mbarrier
     const uint32_t base0 = smem_u32addr(Is0), slab1 = (uint32_t)((size_t)P * NPP * sizeof(C2<T>));
-    for (int z = tid; z < N; z += nt) s_zt[z] = cluster_map(base0 + (uint32_t)((z % P) * NPP * sizeof(C2<T>)), z / P);
+    // the mbarrier of this CTA's slabs: one arrival (the expected bytes) and the bytes themselves per op
+    const uint32_t mbar = smem_u32addr(s_zt + N);
+    uint32_t phase = 0;
+    for (int z = tid; z < N; z += nt)
+        s_zt[z] = make_uint2(cluster_map(base0 + (uint32_t)((z % P) * NPP * sizeof(C2<T>)), z / P), cluster_map(mbar, z / P));
+    if (ASYNC && tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");    // visible behind the first cluster barrier
+    }
 
     const int64_t nclusters = gridDim.x / C;
     const int64_t cid = blockIdx.x / C;
@@ -405,7 +460,8 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                     held = false;
                 }
                 if (has) {
-                    rg_scatter<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
+                    if constexpr (ASYNC) rg_scatter_async<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_at<N>(ky, kx) * 8));
+                    else rg_scatter<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
                     if (a.prefetch && o + 1 < a.nops) {
                         // pull the next op's multipliers of this item towards L1 while the local
                         // passes run (the next op has the same item split: both directions or, after
@@ -418,7 +474,17 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                 }
             }
             if (held) bar.war_wait();      // warps without an item
-            bar.full();
+            if constexpr (ASYNC) {
+                // the peers start the next phase only after this CTA's arrival at the end of the op, so
+                // every byte counts towards the phase that this wait is for
+                if (tid == 0)
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar),
+                                 "r"((uint32_t)((pair ? 2 : 1) * rows * NH * (int)sizeof(C2<T>))) : "memory");
+                if (!slab_wait(mbar, phase)) record_status(a.status, 5);      // EF_ERR_TIMEOUT
+                phase ^= 1;
+            } else {
+                bar.full();
+            }
 
             // ---------------- B: axis 1 inverse on the stored k_x < N/2 columns of each slab
             const int ncol = (pair ? 2 : 1) * P * NH;

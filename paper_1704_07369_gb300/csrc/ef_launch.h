@@ -32,6 +32,14 @@ int tm_maxthreads_f32(int N);
 cudaError_t tm_setup_f32(int N, int v, size_t smem, int cluster, int tpb, int *max_clusters);
 cudaError_t tm_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, cudaStream_t s);
 size_t rg_smem_f32(int N, int planes, int v);
+// variants 1 - 4 by cluster size: scatter behind the cluster barrier (plain) or by st.async
+#define EF_DECLARE_RG(KIND)                                                                            \
+    cudaError_t rg_##KIND##_setup_f32(int N, int v, size_t smem, int cluster, int tpb, int *max_clusters); \
+    cudaError_t rg_##KIND##_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, \
+                                       cudaStream_t s);
+EF_DECLARE_RG(plain)
+EF_DECLARE_RG(async)
+#undef EF_DECLARE_RG
 cudaError_t rg_setup_f32(int N, int v, size_t smem, int cluster, int tpb, int *max_clusters);
 cudaError_t rg_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, cudaStream_t s);
 
