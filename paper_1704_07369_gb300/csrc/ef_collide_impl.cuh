@@ -89,6 +89,24 @@ struct Sync {
     }
 };
 
+template <int V>
+struct IntC {
+    static constexpr int value = V;
+};
+
+// ops [o0, o1) of part prt of a cell split into a.nsplit parts: the units are the ops of a paired list,
+// and the pairs (S set, G add) plus the loss of a single-slab list
+__device__ __forceinline__ void split_range(const CollideArgs &a, int prt, int &o0, int &o1)
+{
+    o0 = 0;
+    o1 = a.nops;
+    if (a.nsplit > 1) {
+        const int per = a.paired ? 1 : 2, units = (a.nops + per - 1) / per;
+        o0 = per * (prt * units / a.nsplit);
+        o1 = min(per * ((prt + 1) * units / a.nsplit), a.nops);
+    }
+}
+
 __device__ __forceinline__ void record_status(int *status, int code)
 {
     if (status) atomicCAS(status, 0, code);
@@ -441,6 +459,55 @@ __device__ __forceinline__ void gather_pencil(C2<T> (&v)[N], C2<T> *slab, int P,
     }
 }
 
+// Per-cell FP64 reduction of the diagnostics: warps by shuffles, the CTA's warps by kDiag threads,
+// the cluster's CTAs by rank 0 (distributed shared memory); full warps.  part: 33 * kDiag doubles.
+template <int D, typename SYNC>
+__device__ __forceinline__ void diag_reduce_f64(const CollideArgs &a, Diag &dg, double *part, int lane, int tid, int nt, int rank,
+                                                int C, SYNC &bar, cg::cluster_group &cl, int64_t cglob)
+{
+    dg.sum[7] = dg.min_f;
+    dg.sum[8] = dg.max_nu;
+    dg.sum[9] = dg.min_out;
+    const int warp = tid >> 5, nw = (nt + 31) >> 5;
+#pragma unroll
+    for (int k = 0; k < kDiag; ++k) {
+        double v = dg.sum[k];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, s);
+            v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
+        }
+        if (lane == 0) part[warp * kDiag + k] = v;
+    }
+    __syncthreads();
+    if (tid < kDiag) {
+        const int k = tid;
+        double v = part[k];
+        for (int w2 = 1; w2 < nw; ++w2) {
+            const double u = part[w2 * kDiag + k];
+            v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
+        }
+        part[32 * kDiag + k] = v;
+    }
+    bar.full();
+    if (rank == 0 && tid < kDiag) {
+        const int k = tid;
+        double v = part[32 * kDiag + k];
+        for (int r = 1; r < C; ++r) {
+            const double *rp = cl.map_shared_rank(part, r);
+            const double u = rp[32 * kDiag + k];
+            v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
+        }
+        const double hd = (D == 3) ? a.h * a.h * a.h : a.h * a.h;
+        if (k == 0 || k == 5) v *= hd;
+        else if (k >= 1 && k <= 3) v *= hd * a.h;
+        else if (k == 4) v *= 0.5 * hd * a.h * a.h;
+        if (D == 2 && k == 3) v = 0.0;
+        a.diag[cglob * kDiag + k] = v;
+    }
+    bar.war();
+}
+
 template <typename T, int D, int N, int OCC = 1>
 __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads, OCC) collide_kernel(const CollideArgs a)
 {
@@ -498,16 +565,27 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
     const T *Mbase = reinterpret_cast<const T *>(a.mult);
 
     const int64_t ncells = a.dev_ncells ? (int64_t)*a.dev_ncells : a.ncells;
-    int64_t c = cid - nclusters;
+    const int S = a.nsplit;                 // parts per cell, each with its share of the ops
+    const int64_t nwork = ncells * S;
+    int64_t w = cid - nclusters;
     for (;;) {
-        if (a.counter) {            // dynamic: the cluster takes the next unclaimed cell
+        if (a.counter) {            // dynamic: the cluster takes the next unclaimed item
             if (rank == 0 && tid == 0) *s_cell = (long long)atomicAdd(a.counter, 1ULL);
             bar.full();
-            c = *cl.map_shared_rank(s_cell, 0);
+            w = *cl.map_shared_rank(s_cell, 0);
         } else {
-            c += nclusters;
+            w += nclusters;
         }
-        if (c >= ncells) break;
+        if (w >= nwork) break;
+        const int64_t c = S > 1 ? w / S : w;
+        const int prt = S > 1 ? (int)(w - c * S) : 0;
+        int o0, o1;
+        split_range(a, prt, o0, o1);
+        T *pnu = nullptr, *pg = nullptr;    // split: nu of the cell, this part's gain
+        if (S > 1) {
+            pnu = reinterpret_cast<T *>(a.part) + (c * (S + 1) + S) * CELL;
+            pg = reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL;
+        }
         const int64_t coff = a.cell_off ? a.cell_off[c] : c * CELL;
         const int64_t cglob = a.cell_id ? a.cell_id[c] : c;
         const T *F = reinterpret_cast<const T *>(a.F) + coff;
@@ -567,8 +645,9 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
 
         Diag dg;
         dg.reset();
+        bool have_g = false;                // split: this part's G is already set
 
-        for (int o = 0; o < a.nops; ++o) {
+        for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
             const bool pair = op.kind >= OP_PAIR;
             // ---------------- A: multiply, inverse along axis 0, scatter to the owners' slabs;
@@ -588,7 +667,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                     for (int z = 0; z < N; ++z) v[z] = cscale(Fh[(size_t)z * NP + pencil], __ldg(M + (size_t)z * NP));
                     fft<N, 1, N>(v);
                     scatter_pencil<T, N, WIDE>(v, b ? Is1 : Is0, P, pm, NPP, pencil, mask);
-                    if (a.prefetch && o + 1 < a.nops) {   // pull the next op's multipliers towards L1
+                    if (a.prefetch && o + 1 < o1) {   // pull the next op's multipliers towards L1
                         const Op nx = a.ops[o + 1];
                         const T *Mn = Mbase + (size_t)(b ? nx.dir2 : nx.dir) * N * NP + pencil;
 #pragma unroll
@@ -618,7 +697,9 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
             if (pair) {
                 // one row per thread, both directions at once: a_e (slab 0) and S_e (slab 1)
                 // come out of a single complex transform; G (column-major) += a_e S_e
-                const bool last = op.kind == OP_PAIR_LAST;
+                const bool last = op.kind == OP_PAIR_LAST && S == 1;
+                const bool fresh = S > 1 && !have_g;
+                have_g = true;
                 const bool big = *s_nubig != 0;
                 for (int r = tid; r < rows; r += nt) {
                     // two Hermitian half rows -> one complex row z (a_e + i S_e), built straight
@@ -627,7 +708,10 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                     const int ro = (r / N1) * NPP + (r % N1) * H;
                     c2r_rows_from<N, T>(Is0 + ro, Is1 + ro, z);
                     T *Gr = Gb + r;
-                    if (!last) {
+                    if (fresh) {
+#pragma unroll
+                        for (int n = 0; n < N; ++n) Gr[n * rows] = z[n].x * z[n].y;
+                    } else if (!last) {
 #pragma unroll
                         for (int n = 0; n < N; ++n) Gr[n * rows] += z[n].x * z[n].y;
                     } else {
@@ -649,15 +733,25 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                     // consecutive rows, so every access below is conflict free without padding
                     T *S0 = Sb + r0, *S1 = Sb + r1;
                     T *G0 = Gb + r0, *G1 = Gb + r1;
-                    const T w = T(op.w);
-                    switch (op.kind) {
+                    const T wt = T(op.w);
+                    int kind = op.kind;
+                    if (S > 1 && kind == OP_G_ADD && !have_g) kind = OP_G_SET;
+                    if (S > 1 && (kind == OP_NU_INIT || kind == OP_LOSS)) {     // nu to the workspace
+                        T nu0[N], nu1[N];
+#pragma unroll
+                        for (int n = 0; n < N; ++n) { nu0[n] = z[n].x; nu1[n] = z[n].y; }
+                        store_row<T, N>(pnu + ((int64_t)rank * rows + r0) * N, nu0);
+                        store_row<T, N>(pnu + ((int64_t)rank * rows + r1) * N, nu1);
+                        continue;
+                    }
+                    switch (kind) {
                     case OP_S_SET:
 #pragma unroll
-                        for (int n = 0; n < N; ++n) { S0[n * rows] = w * z[n].x; S1[n * rows] = w * z[n].y; }
+                        for (int n = 0; n < N; ++n) { S0[n * rows] = wt * z[n].x; S1[n * rows] = wt * z[n].y; }
                         break;
                     case OP_S_ADD:
 #pragma unroll
-                        for (int n = 0; n < N; ++n) { S0[n * rows] += w * z[n].x; S1[n * rows] += w * z[n].y; }
+                        for (int n = 0; n < N; ++n) { S0[n * rows] += wt * z[n].x; S1[n * rows] += wt * z[n].y; }
                         break;
                     case OP_G_SET:
 #pragma unroll
@@ -710,54 +804,26 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                     } break;
                     }
                 }
+                if (op.kind == OP_G_SET || op.kind == OP_G_ADD) have_g = true;
             }
             bar.war();
         }
 
-        // ---------------- per-cell FP64 reduction of the diagnostics
-        if (a.diag) {
-            dg.sum[7] = dg.min_f;
-            dg.sum[8] = dg.max_nu;
-            dg.sum[9] = dg.min_out;
-            const int lane = tid & 31, warp = tid >> 5, nw = (nt + 31) >> 5;
-#pragma unroll
-            for (int k = 0; k < kDiag; ++k) {
-                double v = dg.sum[k];
-#pragma unroll
-                for (int s = 16; s > 0; s >>= 1) {
-                    const double u = __shfl_xor_sync(0xffffffffu, v, s);
-                    v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
-                }
-                if (lane == 0) part[warp * kDiag + k] = v;
-            }
+        if (S > 1) {
+            // this part's gain (a part with only the loss leaves zeros)
             __syncthreads();
-            if (tid < kDiag) {
-                const int k = tid;
-                double v = part[k];
-                for (int w2 = 1; w2 < nw; ++w2) {
-                    const double u = part[w2 * kDiag + k];
-                    v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
-                }
-                part[32 * kDiag + k] = v;
+            for (int r = tid; r < rows; r += nt) {
+                T g[N];
+#pragma unroll
+                for (int n = 0; n < N; ++n) g[n] = have_g ? Gb[r + (size_t)n * rows] : T(0);
+                store_row<T, N>(pg + ((int64_t)rank * rows + r) * N, g);
             }
-            bar.full();
-            if (rank == 0 && tid < kDiag) {
-                const int k = tid;
-                double v = part[32 * kDiag + k];
-                for (int r = 1; r < C; ++r) {
-                    const double *rp = cl.map_shared_rank(part, r);
-                    const double u = rp[32 * kDiag + k];
-                    v = (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u);
-                }
-                const double hd = (D == 3) ? a.h * a.h * a.h : a.h * a.h;
-                if (k == 0 || k == 5) v *= hd;
-                else if (k >= 1 && k <= 3) v *= hd * a.h;
-                else if (k == 4) v *= 0.5 * hd * a.h * a.h;
-                if (D == 2 && k == 3) v = 0.0;
-                a.diag[cglob * kDiag + k] = v;
-            }
-            bar.war();
+            __syncthreads();                // G is rewritten by the next item
+            continue;
         }
+
+        // ---------------- per-cell FP64 reduction of the diagnostics
+        if (a.diag) diag_reduce_f64<D>(a, dg, part, lane, tid, nt, rank, C, bar, cl, cglob);
     }
     bar.war();   // no CTA leaves while a peer may still read its shared memory
 }

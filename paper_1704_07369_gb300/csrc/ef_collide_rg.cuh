@@ -309,7 +309,7 @@ __device__ __forceinline__ void diag_reduce_cell(const CollideArgs &a, const Dia
 
 // GS = false: G of this thread's RPT rows in registers (nt * RPT = rows); GS = true: G in shared
 // memory, column-major ([x][row], so consecutive threads touch consecutive banks), rows looped.
-template <int D, int N, int RPT, int LB, bool GS, bool ASYNC>
+template <int D, int N, int RPT, int LB, bool GS, bool ASYNC, bool SPLIT = false>
 __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
 {
     static_assert(D == 3, "3D only");
@@ -364,20 +364,27 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
     constexpr int NPT = N * H;             // multiplier table: [dir][k_z][k_y * H + k_x]
 
     const int64_t ncells = a.dev_ncells ? (int64_t)*a.dev_ncells : a.ncells;
-    int64_t c = cid - nclusters;
+    const int S = SPLIT ? a.nsplit : 1;    // parts per cell, each with its share of the ops
+    const int64_t nwork = ncells * S;
+    int64_t w = cid - nclusters;
     for (;;) {
         if (a.counter) {
             if (rank == 0 && tid == 0) *s_cell = (long long)atomicAdd(a.counter, 1ULL);
             bar.full();
-            c = *cl.map_shared_rank(s_cell, 0);
+            w = *cl.map_shared_rank(s_cell, 0);
         } else {
-            c += nclusters;
+            w += nclusters;
         }
-        if (c >= ncells) break;
+        if (w >= nwork) break;
+        const int64_t c = S > 1 ? w / S : w;
+        const int prt = S > 1 ? (int)(w - c * S) : 0;
+        int o0 = 0, o1 = a.nops;
+        if (SPLIT) split_range(a, prt, o0, o1);
         const int64_t coff = a.cell_off ? a.cell_off[c] : c * CELL;
         const int64_t cglob = a.cell_id ? a.cell_id[c] : c;
         const T *F = reinterpret_cast<const T *>(a.F) + coff;
         T *Out = reinterpret_cast<T *>(a.Q) + coff;
+        T *pnu = reinterpret_cast<T *>(a.part) + (c * (S + 1) + S) * CELL;       // split: the cell's nu
         if (tid == 0) *s_nubig = 0;
 
         // ---------------- F1: own rows real -> half complex (k_x < N/2 kept), two rows per item
@@ -430,13 +437,24 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
         DiagF dg;
         T g[GS ? 1 : RPT][N];              // G in registers: this thread's rows tid + j nt
 
-        for (int o = 0; o < a.nops; ++o) {
+        if (S > 1) {
+            if constexpr (GS) {
+                for (int i = tid; i < rows * N; i += nt) Gs[i] = T(0);       // read after later barriers
+            } else {
+#pragma unroll
+                for (int j = 0; j < RPT; ++j)
+#pragma unroll
+                    for (int n = 0; n < N; ++n) g[j][n] = T(0);
+            }
+        }
+
+        for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
             const bool pair = op.kind >= OP_PAIR;
             // ---------------- A: multiply, axis 0 inverse, scatter (one (direction, pencil) item
             // per thread; lanes of a pair share the direction since NPC is even)
             const int nitems = (pair ? 2 : 1) * NPC;
-            bool held = o > 0;             // the previous op's slabs are not yet known to be read by all
+            bool held = o > o0;            // the previous op's slabs are not yet known to be read by all
             for (int q0 = tid - lane; q0 < nitems; q0 += nt) {
                 const int qi = q0 + lane;
                 const bool has = qi < nitems;
@@ -462,7 +480,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                 if (has) {
                     if constexpr (ASYNC) rg_scatter_async<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_at<N>(ky, kx) * 8));
                     else rg_scatter<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
-                    if (a.prefetch && o + 1 < a.nops) {
+                    if (a.prefetch && o + 1 < o1) {
                         // pull the next op's multipliers of this item towards L1 while the local
                         // passes run (the next op has the same item split: both directions or, after
                         // the loss, two); a hint only, every address is inside the table
@@ -504,7 +522,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
 
             // ---------------- rows: half complex -> real, accumulate / output
             if (pair) {
-                const bool last = op.kind == OP_PAIR_LAST;
+                const bool last = op.kind == OP_PAIR_LAST && S == 1;
                 const bool big = *s_nubig != 0;
                 if (last) dg.reset();
                 if constexpr (GS) {
@@ -565,6 +583,12 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         for (int j = 0; j < 2; ++j) {
                             const int r = j ? r1 : r0;
                             T fr[N];
+                            if (S > 1) {
+#pragma unroll
+                                for (int n = 0; n < N; ++n) fr[n] = j ? z[n].y : z[n].x;
+                                store_row<T, N>(pnu + ((int64_t)rank * rows + r) * N, fr);
+                                continue;
+                            }
                             load_row<T, N>(F + ((int64_t)rank * rows + r) * N, fr);
                             T mx = j ? z[0].y : z[0].x;
 #pragma unroll
@@ -597,6 +621,12 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         z[NH] = C2<T>{0.f, 0.f};
                         fft<N, 1, N>(z);
                         T fr[N];
+                        if (S > 1) {
+#pragma unroll
+                            for (int n = 0; n < N; ++n) fr[n] = z[n].x;
+                            store_row<T, N>(pnu + ((int64_t)rank * rows + r) * N, fr);
+                            continue;
+                        }
                         load_row<T, N>(F + ((int64_t)rank * rows + r) * N, fr);
                         T mx = z[0].x;
 #pragma unroll
@@ -619,7 +649,25 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             }
             // write-after-read: the next op's scatter waits for this arrival
             bar.war_arrive();
-            if (o + 1 == a.nops) bar.war_wait();
+            if (o + 1 == o1) bar.war_wait();
+        }
+
+        if (S > 1) {                       // this part's gain (zeros from a part with only the loss)
+            T *pg = reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL + (int64_t)rank * rows * N;
+            if constexpr (GS) {
+                __syncthreads();
+                for (int r = tid; r < rows; r += nt) {
+                    T gv[N];
+#pragma unroll
+                    for (int n = 0; n < N; ++n) gv[n] = Gs[n * rows + r];
+                    store_row<T, N>(pg + (int64_t)r * N, gv);
+                }
+                __syncthreads();
+            } else {
+#pragma unroll
+                for (int j = 0; j < RPT; ++j) store_row<T, N>(pg + (int64_t)(tid + j * nt) * N, g[j]);
+            }
+            continue;
         }
 
         // ---------------- per-cell reduction of the diagnostics

@@ -58,7 +58,10 @@ struct CollideArgs {
     int paired;               // 1: two spectral slabs per CTA and the paired op kinds
     const long long *dev_ncells;  // nullable: cell count read from device memory at kernel start
     void *fh_ws;              // forward spectrum workspace: per cluster slot N * NP complex, [z][p]
-    int npc;                  // axis-0 pencils per CTA (even; CTA r owns [r npc, (r + 1) npc) of NP)
+    int npc;                  // axis-0 pencils per CTA (CTA r owns [r npc, (r + 1) npc) of NP)
+    int nsplit = 1;           // parts per cell (>= 1): a work item is one part, with its share of the ops
+    void *part = nullptr;     // nsplit > 1: [cell][nsplit + 1][N^d] gain of each part, then nu; summed and
+                              // written out by the finishing kernel (ef_split.cu)
 };
 
 // Arguments of the low-mode feature kernel (one launch per size class).

@@ -42,6 +42,12 @@ EF_DECLARE_RG(async)
 #undef EF_DECLARE_RG
 cudaError_t rg_setup_f32(int N, int v, size_t smem, int cluster, int tpb, int *max_clusters);
 cudaError_t rg_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, cudaStream_t s);
+// the split instantiations of variants 1 and 2 (ef_collide_rg_split_f32.cu)
+cudaError_t rg_split_setup_f32(int N, int v, size_t smem, int cluster, int tpb, int *max_clusters);
+cudaError_t rg_split_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, cudaStream_t s);
+// Q / F + dt Q and diagnostics from the parts of a split collide launch (ef_split.cu)
+cudaError_t split_finish_setup(int prec, int d);
+cudaError_t split_finish_launch(int prec, int d, int N, const CollideArgs &a, cudaStream_t s);
 
 EF_DECLARE_VARIANT(f32_2d)
 EF_DECLARE_VARIANT(f32_3d)
@@ -68,6 +74,9 @@ struct PlanView {
 };
 bool plan_view(const struct ef_plan_s *p, PlanView *out);
 // uniform plan on the doubled grid 2N with multipliers restricted to the N grid's Galerkin modes
+// ef_plan_create_batched; may_split = false for plans whose steps run side by side on several streams
+ef_status ef_plan_create_batched_opt(int d, int64_t ncells, const int *N_host, double L, ef_kernel kernel, int R, ef_precision prec,
+                              bool may_split, struct ef_plan_s **out);
 ef_status plan_create_padded(const ef_plan_desc *desc, struct ef_plan_s **out);
 
 // Axis-0 pencils per CTA of a C-CTA cluster (even, so that lane pairs never straddle CTAs) and the
@@ -87,7 +96,8 @@ size_t collide_smem(int prec, int d, int N, int planes, int sg_global, int paire
 // 3 / 4 / 5 / 6 = FP32 3D kernel that keeps the forward spectrum in shared memory and skips the
 // Nyquist column (pencils: N^2 / (2 C) per CTA), with the gain accumulator in registers (one row
 // per thread / two / one with at most 200 threads) or (6) in shared memory.
-inline int collide_npc_v(int d, int N, int C, int occ)
+// FP64 (prec 1): the team kernel, which drops the Nyquist column too.
+inline int collide_npc_v(int prec, int d, int N, int C, int occ)
 {
     if (occ >= 3) {
         const int np = N * N / 2;

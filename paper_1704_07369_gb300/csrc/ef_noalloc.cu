@@ -127,7 +127,7 @@ extern "C" ef_status ef_collide_noalloc(ef_plan_t plan, const void *F_dev, void 
     a.sg_global = onchip ? 0 : 1;
     a.sg_ws = static_cast<unsigned char *>(base) + kCounterBytes;
     a.fh_ws = static_cast<unsigned char *>(base) + kCounterBytes + (size_t)grid * v.cluster * per_cta;
-    a.npc = ef::collide_npc_v(v.d, v.N, v.cluster, v.occ);
+    a.npc = ef::collide_npc_v(v.prec, v.d, v.N, v.cluster, v.occ);
     a.out_mode = ef::OUT_COLLIDE;
     a.h = 2.0 * v.L / v.N;
     a.status = v.status;

@@ -20,6 +20,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <string>
 #include <thread>
 #include <vector>
@@ -240,11 +241,26 @@ int mode_of(int N, int i) { return i < N / 2 ? i : i - N; }
 
 // ---------------------------------------------------------------- plan objects -------------
 
+struct Shape {
+    int cluster, tpb, planes, sg_global, paired, occ;
+    size_t smem;
+    int max_clusters;
+};
+
 struct ClassPlan {
     int N = 0;
     int64_t ncells = 0;                 // batched: cells of this size; uniform plan: 0
     int cluster = 1, tpb = 32, planes = 0, sg_global = 0, prefetch = 1, paired = 0, occ = 1;
     double tuned_ms = 0.0;              // autotuner's best time (0 when not tuned)
+    int split = 1;                      // batched: parts per cell of every launch
+    Shape cur{};                        // the shape of the fields above
+    std::vector<Shape> shapes;          // uniform: the shapes a call may choose from by its cell count
+    int pin_split = 0;                  // > 0: parts per cell pinned with the shape
+    int64_t pick_n = -1;                // the last choice: cell count, shape, parts
+    size_t pick_i = 0;
+    int pick_s = 1;
+    void *d_part = nullptr;             // gains of the parts of split launches, kPartSlots workspaces
+    size_t part_bytes = 0;              // of one workspace
     size_t smem = 0;
     int max_clusters = 0;
     int ndir = 0, nops = 0;              // op count of the active mode
@@ -263,6 +279,27 @@ struct ClassPlan {
 
 }  // namespace
 
+// Part workspaces of a plan: 0 for calls, the rest for callers' stream captures.  A graph may be replayed
+// beside anything, so the split calls captured on one stream of one capture take a workspace that no
+// other graph uses, and give it back when the graph and its executables are destroyed (a user object
+// that the graph retains).  With none left a captured call is not split.
+constexpr int kPartSlots = 5;
+struct PartSlots {
+    std::atomic<int> taken[kPartSlots]{};
+    unsigned long long capture[kPartSlots]{};
+    cudaStream_t stream[kPartSlots]{};      // of the capture that holds the workspace
+};
+struct PartLease {
+    std::shared_ptr<PartSlots> slots;
+    int i;
+};
+void CUDART_CB end_lease(void *p)
+{
+    PartLease *l = static_cast<PartLease *>(p);
+    l->slots->taken[l->i].store(0);
+    delete l;
+}
+
 struct ef_plan_s {
     Desc desc;
     // concurrent size classes: one internal stream, event and cell counter per class
@@ -272,6 +309,8 @@ struct ef_plan_s {
     unsigned long long *d_counters = nullptr;
     int device = 0;
     bool batched = false;
+    bool may_split = true;              // launches may split cells into parts (off for plans that run side by side)
+    int sms = 1;
     int64_t ncells = 0;
     std::vector<ClassPlan> classes;
     int64_t *d_all_off = nullptr, *d_all_N = nullptr;
@@ -286,7 +325,13 @@ struct ef_plan_s {
     int g_mode = -1;
     double g_dt = 0.0;
     double *g_diag = nullptr;
+    int g_slot = -1;
     cudaStream_t g_stream = nullptr;
+    // split launches share the part workspace 0: an event behind the last one, which the next waits for
+    // (nothing to wait for on the same stream); captured calls have workspaces 1 .. of their graphs
+    cudaEvent_t split_done = nullptr;
+    bool split_used = false;
+    std::shared_ptr<PartSlots> slots;
     // SSP-RK3 stage buffers: two batch-sized arrays, grown on demand
     void *d_rk = nullptr;
     size_t rk_bytes = 0;
@@ -330,11 +375,15 @@ cudaError_t launch_for(int prec, int d, int N, const ef::CollideArgs &a, int gri
                   : ef::collide_launch_f64_2d(N, a, grid, tpb, smem, occ, s);
 }
 
-struct Shape {
-    int cluster, tpb, planes, sg_global, paired, occ;
-    size_t smem;
-    int max_clusters;
-};
+// One class launch in shape sh, with the finishing launch of a split one behind it.
+cudaError_t launch_shape(const Desc &ds, int N, const ef::CollideArgs &a, int grid, const Shape &sh, cudaStream_t s)
+{
+    const bool rg = ds.prec == EF_PREC_F32 && ds.d == 3 && sh.occ >= 3;
+    if (a.nsplit <= 1) return launch_for(ds.prec, ds.d, N, a, grid, sh.tpb, sh.smem, sh.occ, s);
+    cudaError_t e = rg ? ef::rg_split_launch_f32(N, sh.occ - 2, a, grid, sh.tpb, sh.smem, s)
+                       : launch_for(ds.prec, ds.d, N, a, grid, sh.tpb, sh.smem, sh.occ, s);
+    return e != cudaSuccess ? e : ef::split_finish_launch(ds.prec == EF_PREC_F32 ? 0 : 1, ds.d, N, a, s);
+}
 
 // Every launch shape that fits one N: cluster sizes C | N with an even number of real rows per
 // CTA; threads per CTA enough for one work item each of the widest stage (the stage-A (direction,
@@ -354,7 +403,7 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
     // FP32 3D: the register-accumulator kernel first (one or two rows per thread, threads = rows / RPT)
     if (ds.prec == EF_PREC_F32 && d == 3) {
         for (int C : cands) {
-            if (N % C || ef::collide_npc_v(d, N, C, 3) == 0) continue;
+            if (N % C || ef::collide_npc_v(0, d, N, C, 3) == 0) continue;
             const int planes = N / C, rows = planes * N;
             for (int v = 1; v <= 6; ++v) {
                 const int occ = 2 + v;
@@ -377,6 +426,15 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
                         continue;
                     }
                     if (mc <= 0) continue;
+                    if (occ <= 4) {        // also built split: the same shape, perhaps other registers
+                        int ms = 0;
+                        e = ef::rg_split_setup_f32(N, v, smem, C, tpb, &ms);
+                        if (e != cudaSuccess || ms <= 0) {
+                            cudaGetLastError();
+                            continue;
+                        }
+                        mc = std::min(mc, ms);
+                    }
                     out.push_back(Shape{C, tpb, planes, 0, 1, occ, smem, mc});
                 }
             }
@@ -391,14 +449,19 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
                 const int rows = planes * N1;
                 if (rows % 2) continue;
                 const int nb = paired ? 2 : 1;
-                const int need = std::max({nb * ef::collide_npc(d, N, C), paired ? rows : rows / 2,
-                                           d == 3 ? nb * planes * H : 1});
+                // FP64: four lanes per line, N/2 stored columns (ef_collide_q.cuh)
+                const bool quad = false;
+                const int need = quad ? 4 * std::max({nb * ef::collide_npc_v(1, d, N, C, 1), paired ? rows : rows / 2,
+                                                      d == 3 ? nb * planes * (N / 2) : 1})
+                                      : std::max({nb * ef::collide_npc(d, N, C), paired ? rows : rows / 2,
+                                                  d == 3 ? nb * planes * H : 1});
                 const size_t smem = smem_for(ds.prec, d, N, planes, sg, paired, 1);
                 if ((long)smem > smem_max) continue;
                 for (int occ = 1; occ <= 2; ++occ) {
                     const int tmax = maxthreads_for(ds.prec, d, N, occ);
                     int last = 0;
-                    for (int rounds = 1; rounds <= 2; ++rounds) {
+                    const int rounds0 = quad && tmax ? (need + tmax - 1) / tmax : 1;
+                    for (int rounds = rounds0; rounds <= 2 * rounds0; rounds += rounds0) {
                         const int tpb = std::max(64, ((need + rounds - 1) / rounds + 31) / 32 * 32);
                         if (tpb > tmax || tpb == last) continue;
                         last = tpb;
@@ -419,6 +482,83 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
     return out;
 }
 
+// Parts per cell a launch of n cells may use: all its items resident at once, at most one part per unit
+// (a pair of transforms, or the loss), and only the kernels built for it.
+int units_of(const ClassPlan &cp) { return (cp.nops_paired > 0 ? cp.nops_paired : 1); }
+
+int max_split(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64_t n)
+{
+    if (ds.prec == EF_PREC_F32 && ds.d == 3 && sh.occ != 1 && sh.occ != 3 && sh.occ != 4) return 1;
+    if (n <= 0 || n >= sh.max_clusters) return 1;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(units_of(cp), sh.max_clusters / n));
+}
+
+// Estimated SM cycles of one launch of n cells in shape sh with S parts per cell: the waves of items,
+// each a forward transform and its share of the units, one unit three line passes (two in 2D).
+//   FP32: a pass is bound by issue (about 3 cycles an instruction and warp on a sub-partition) or, with
+//   few warps, by latency (5.5 cycles an instruction); a line takes about 9 N log2 N / 3 instructions
+//   with its loads and stores.
+//   FP64: one warp instruction of the FP64 pipe per 64 cycles and sub-partition, (3 log2 N + 2) N / 4 of
+//   them per lane and line.
+// The constants are the rates that the kernels showed (ncu, FP32 N = 32 - 64; FP64 pipe rate); the model
+// only ranks shapes.
+double launch_cycles(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64_t n, int S, int sms)
+{
+    const int N = cp.N, d = ds.d, passes = d;
+    const double lg = std::log2((double)N);
+    const int64_t items = n * S;
+    const int64_t live = std::min<int64_t>(items, sh.max_clusters);
+    const double waves = (double)((items + sh.max_clusters - 1) / sh.max_clusters);
+    const int per_sm = (int)std::max<int64_t>(1, (live * sh.cluster + sms - 1) / sms);      // CTAs sharing an SM
+    const int rows = sh.planes * (d == 3 ? N : 1);
+    double pass;
+    if (ds.prec == EF_PREC_F64) {
+        const int warps = (rows * 4 + 31) / 32;
+        pass = (double)((warps * per_sm + 3) / 4) * (3.0 * lg + 2.0) * N / 4 * 64.0 + 1000.0;
+    } else {
+        const double instr = 3.0 * N * lg;
+        const int rounds = (rows + sh.tpb - 1) / sh.tpb;
+        const double warps = (double)std::min(rows, sh.tpb) / 32.0 * per_sm / 4.0;
+        pass = rounds * instr * std::max(5.5, 3.0 * std::max(1.0, warps)) + 300.0;
+    }
+    const double unit = passes * pass + (sh.cluster > 1 ? 1500.0 + 100.0 * sh.cluster : 500.0) / per_sm;
+    const int units = units_of(cp);
+    double t = waves * unit * (1.0 + (units + S - 1) / S);
+    if (S > 1) {
+        const double bytes = (double)n * (S + 3) * std::pow((double)N, d) * (ds.prec == EF_PREC_F64 ? 8 : 4);
+        t += 12000.0 + bytes / 2000.0;      // the finishing launch and the event wait: about 6 us; 4 TB/s
+    }
+    return t;
+}
+
+// The shape and parts of a call on n cells of a uniform plan.  The plan's first shape (the smallest
+// cluster that fits) is kept unless another one, or a split, is estimated at least a tenth faster.
+void pick_shape(const Desc &ds, ClassPlan &cp, int64_t n, int sms)
+{
+    if (cp.pick_n == n) return;
+    cp.pick_n = n;
+    cp.pick_i = 0;
+    cp.pick_s = 1;
+    if (cp.pin_split > 0) {
+        cp.pick_s = std::min(cp.pin_split, max_split(ds, cp, cp.shapes[0], n));
+        return;
+    }
+    double tb = 0.9 * launch_cycles(ds, cp, cp.shapes[0], n, 1, sms);
+    const int u = units_of(cp);
+    for (size_t i = 0; i < cp.shapes.size(); ++i) {
+        const int sm = max_split(ds, cp, cp.shapes[i], n);
+        for (int k = 1; k <= sm; ++k) {
+            if (k > 1 && (u + k - 1) / k == (u + k - 2) / (k - 1)) continue;      // no shorter longest part
+            const double t = launch_cycles(ds, cp, cp.shapes[i], n, k, sms);
+            if (t < tb) {
+                tb = t;
+                cp.pick_i = i;
+                cp.pick_s = k;
+            }
+        }
+    }
+}
+
 void apply_shape(ClassPlan &cp, const Shape &sh)
 {
     cp.cluster = sh.cluster;
@@ -429,6 +569,7 @@ void apply_shape(ClassPlan &cp, const Shape &sh)
     cp.occ = sh.occ;
     cp.smem = sh.smem;
     cp.max_clusters = sh.max_clusters;
+    cp.cur = sh;
     cp.d_ops = sh.paired ? cp.d_ops_paired : cp.d_ops_single;
     cp.nops = sh.paired ? cp.nops_paired : cp.nops_single;
 }
@@ -453,13 +594,13 @@ std::string tune_key(const Desc &ds, int N, int64_t ncells)
     char buf[256];
     int bucket = 64;
     while (bucket < 4096 && bucket < ncells) bucket *= 4;
-    // "v5": kernel layout generation (variants 3 - 8: register-accumulator kernels, 7 / 8 the team ones)
-    std::snprintf(buf, sizeof(buf), "v5 %s p%d d%d N%d k%d R%d J%d a%d.%d.%d s%d b%d", device_key().c_str(), (int)ds.prec,
+    // "v6": kernel layout generation (variants 3 - 8: register-accumulator kernels, 7 / 8 the team ones)
+    std::snprintf(buf, sizeof(buf), "v6 %s p%d d%d N%d k%d R%d J%d a%d.%d.%d s%d b%d", device_key().c_str(), (int)ds.prec,
                   ds.d, N, (int)ds.kernel, ds.R, ds.J, ds.nmu, ds.nphi, ds.nc, ds.sigma, bucket);
     return buf;
 }
 
-bool cache_lookup(const std::string &key, int &C, int &tpb, int &sg, int &pf, int &pr, int &occ)
+bool cache_lookup(const std::string &key, int &C, int &tpb, int &sg, int &pf, int &pr, int &occ, int &parts)
 {
     const char *path = std::getenv("EF_AUTOTUNE_CACHE");
     if (!path) return false;
@@ -471,19 +612,19 @@ bool cache_lookup(const std::string &key, int &C, int &tpb, int &sg, int &pf, in
         std::string ln(line);
         const size_t bar = ln.find('|');
         if (bar == std::string::npos || ln.substr(0, bar) != key) continue;
-        if (std::sscanf(ln.c_str() + bar + 1, "%d %d %d %d %d %d", &C, &tpb, &sg, &pf, &pr, &occ) == 6) found = true;
+        if (std::sscanf(ln.c_str() + bar + 1, "%d %d %d %d %d %d %d", &C, &tpb, &sg, &pf, &pr, &occ, &parts) == 7) found = true;
     }
     std::fclose(f);
     return found;
 }
 
-void cache_store(const std::string &key, int C, int tpb, int sg, int pf, int pr, int occ, double ms)
+void cache_store(const std::string &key, int C, int tpb, int sg, int pf, int pr, int occ, int parts, double ms)
 {
     const char *path = std::getenv("EF_AUTOTUNE_CACHE");
     if (!path) return;
     FILE *f = std::fopen(path, "a");
     if (!f) return;
-    std::fprintf(f, "%s|%d %d %d %d %d %d %.4f\n", key.c_str(), C, tpb, sg, pf, pr, occ, ms);
+    std::fprintf(f, "%s|%d %d %d %d %d %d %d %.4f\n", key.c_str(), C, tpb, sg, pf, pr, occ, parts, ms);
     std::fclose(f);
 }
 
@@ -493,7 +634,7 @@ void cache_store(const std::string &key, int C, int tpb, int sg, int pf, int pr,
 // on the SMs depend on it), and keep the fastest of those.  Results are cached per device and
 // discretisation in the file named by EF_AUTOTUNE_CACHE when it is set; EF_AUTOTUNE=0 skips the
 // timing and takes the smallest cluster.
-ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
+ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool may_split)
 {
     std::string why;
     std::vector<Shape> shapes = candidate_shapes(ds, cp.N, why);
@@ -501,7 +642,11 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
         return fail(EF_ERR_UNSUPPORTED, "no launch shape fits N=" + std::to_string(cp.N) + " on this device " + why);
     apply_shape(cp, shapes[0]);
     cp.prefetch = 0;
-    // EF_SHAPE="N:cluster:threads:variant[,...]" pins the launch shape of size N (tests, experiments);
+    // a uniform plan's call chooses by its cell count: the first shape, and for the register kernels the
+    // instantiations that can be split
+    for (const Shape &sh : shapes)
+        if (cp.shapes.empty() || cp.shapes[0].occ < 3 || sh.occ == 3 || sh.occ == 4) cp.shapes.push_back(sh);
+    // EF_SHAPE="N:cluster:threads:variant[:parts][,...]" pins the launch shape of size N (tests, experiments);
     // an entry that matches no candidate shape is ignored
     if (const char *pin = std::getenv("EF_SHAPE")) {
         std::string spec(pin);
@@ -509,11 +654,14 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
         while (pos < spec.size()) {
             size_t end = spec.find(',', pos);
             if (end == std::string::npos) end = spec.size();
-            int n = 0, C = 0, tpb = 0, occ = 0;
-            if (std::sscanf(spec.substr(pos, end - pos).c_str(), "%d:%d:%d:%d", &n, &C, &tpb, &occ) == 4 && n == cp.N) {
+            int n = 0, C = 0, tpb = 0, occ = 0, parts = 1;
+            if (std::sscanf(spec.substr(pos, end - pos).c_str(), "%d:%d:%d:%d:%d", &n, &C, &tpb, &occ, &parts) >= 4 && n == cp.N) {
                 for (const Shape &sh : shapes)
                     if (sh.cluster == C && sh.tpb == tpb && sh.occ == occ && sh.sg_global == 0) {
                         apply_shape(cp, sh);
+                        cp.shapes.assign(1, sh);
+                        cp.pin_split = std::max(1, parts);
+                        cp.split = std::min(cp.pin_split, max_split(ds, cp, sh, cp.ncells));
                         return EF_OK;
                     }
             }
@@ -523,20 +671,22 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
     const char *env = std::getenv("EF_AUTOTUNE");
     const bool tune = ncells_tune > 0 && !(env && env[0] == '0') && shapes.size() > 1;
     if (!tune) return EF_OK;
-    const std::string key = tune_key(ds, cp.N, ncells_tune);
-    int C = 0, tpb = 0, sg = 0, pf = 1, pr = 0, occ = 1;
-    if (cache_lookup(key, C, tpb, sg, pf, pr, occ)) {
+    const std::string key = tune_key(ds, cp.N, ncells_tune) + (may_split ? "" : " unsplit");
+    int C = 0, tpb = 0, sg = 0, pf = 1, pr = 0, occ = 1, parts = 1;
+    if (cache_lookup(key, C, tpb, sg, pf, pr, occ, parts)) {
         for (const Shape &sh : shapes)
             if (sh.cluster == C && sh.tpb == tpb && sh.sg_global == sg && sh.paired == pr && sh.occ == occ) {
                 apply_shape(cp, sh);
                 cp.prefetch = pf;
+                // the key's bucket holds other cell counts: at most the parts this count allows
+                cp.split = may_split ? std::max(1, std::min(parts, max_split(ds, cp, sh, ncells_tune))) : 1;
                 return EF_OK;
             }
     }
     const int d = ds.d;
     const int64_t cell = d == 3 ? (int64_t)cp.N * cp.N * cp.N : (int64_t)cp.N * cp.N;
     const size_t el = ds.prec == EF_PREC_F32 ? 4 : 8;
-    void *F = nullptr, *Q = nullptr, *sgws = nullptr, *fhws = nullptr;
+    void *F = nullptr, *Q = nullptr, *sgws = nullptr, *fhws = nullptr, *parts_ws = nullptr;
     double *dgws = nullptr;
     cudaStream_t st = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -545,22 +695,33 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
     if (e == cudaSuccess) e = cudaMemset(F, 0, ncells_tune * cell * el);
     if (e == cudaSuccess) e = cudaMalloc((void **)&dgws, (size_t)ncells_tune * ef::kDiag * sizeof(double));
     int64_t fh_need = 0;
-    for (const Shape &sh : shapes) fh_need = std::max<int64_t>(fh_need, std::min<int64_t>(ncells_tune, sh.max_clusters));
+    // clusters a timed launch may have: a split one has an item for every part
+    auto clusters_of = [&](const Shape &sh) {
+        return std::min<int64_t>(ncells_tune * (may_split ? max_split(ds, cp, sh, ncells_tune) : 1), sh.max_clusters);
+    };
+    for (const Shape &sh : shapes) fh_need = std::max<int64_t>(fh_need, clusters_of(sh));
     if (e == cudaSuccess) e = cudaMalloc(&fhws, (size_t)fh_need * ef::collide_fh_bytes(ds.prec, d, cp.N));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    int64_t part_cells = 0;
+    if (may_split)
+        for (const Shape &sh : shapes) {
+            const int S = max_split(ds, cp, sh, ncells_tune);
+            if (S > 1) part_cells = std::max<int64_t>(part_cells, ncells_tune * (S + 1));
+        }
+    if (e == cudaSuccess && part_cells) e = cudaMalloc(&parts_ws, (size_t)part_cells * cell * el);
     double best = 1e30;
     Shape best_sh = shapes[0];
-    int best_pf = 0;
+    int best_pf = 0, best_split = 1;
     struct Timed {
         double ms;
         size_t shape;
-        int pf;
+        int pf, split;
     };
     std::vector<Timed> sweep;
-    auto time_one = [&](const Shape &sh, int pfv, int64_t nc, double &tmin) -> cudaError_t {
-        const int grid = (int)std::min<int64_t>(nc, sh.max_clusters);
+    auto time_one = [&](const Shape &sh, int pfv, int split, int64_t nc, double &tmin) -> cudaError_t {
+        const int grid = (int)std::min<int64_t>(nc * split, sh.max_clusters);
         ef::CollideArgs a{};
         a.F = F;
         a.Q = Q;
@@ -574,7 +735,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
         a.sg_global = sh.sg_global;
         a.sg_ws = sgws;
         a.fh_ws = fhws;
-        a.npc = ef::collide_npc_v(d, cp.N, sh.cluster, sh.occ);
+        a.npc = ef::collide_npc_v(ds.prec, d, cp.N, sh.cluster, sh.occ);
         // timed as the step runs it: the Euler output in place (dt = 0 leaves F unchanged) with the
         // per-cell diagnostics, which cost some shapes more than others
         a.Q = F;
@@ -583,11 +744,13 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
         a.diag = dgws;
         a.h = 1.0;
         a.prefetch = pfv;
+        a.nsplit = split;
+        a.part = parts_ws;
         tmin = 1e30;
         cudaError_t r = cudaSuccess;
         for (int rep = 0; rep < 4 && r == cudaSuccess; ++rep) {
             r = cudaEventRecord(e0, st);
-            if (r == cudaSuccess) r = launch_for(ds.prec, d, cp.N, a, grid, sh.tpb, sh.smem, sh.occ, st);
+            if (r == cudaSuccess) r = launch_shape(ds, cp.N, a, grid, sh, st);
             if (r == cudaSuccess) r = cudaEventRecord(e1, st);
             if (r == cudaSuccess) r = cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -599,7 +762,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
     const int64_t n1 = std::min<int64_t>(ncells_tune, 512);
     for (size_t i = 0; e == cudaSuccess && i < shapes.size(); ++i) {
         const Shape &sh = shapes[i];
-        const int grid = (int)std::min<int64_t>(ncells_tune, sh.max_clusters);
+        const int grid = (int)clusters_of(sh);
         if (sh.sg_global) {
             const int64_t rows = (int64_t)sh.planes * (d == 3 ? cp.N : 1);
             cudaFree(sgws);
@@ -607,16 +770,18 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
             e = cudaMalloc(&sgws, (size_t)grid * sh.cluster * 2 * rows * cp.N * el);
             if (e != cudaSuccess) break;
         }
-        for (int pfv = 0; pfv <= 1 && e == cudaSuccess; ++pfv) {
+        const int smax = may_split ? max_split(ds, cp, sh, ncells_tune) : 1;
+        for (int v = 0; v < (smax > 1 ? 4 : 2) && e == cudaSuccess; ++v) {
+            const int pfv = v & 1, split = v >= 2 ? smax : 1;
             double tmin = 1e30;
-            e = time_one(sh, pfv, n1, tmin);
+            e = time_one(sh, pfv, split, n1, tmin);
             if (e != cudaSuccess) break;
-            sweep.push_back(Timed{tmin, i, pfv});
+            sweep.push_back(Timed{tmin, i, pfv, split});
             // EF_AUTOTUNE_LOG names a file that receives every timed candidate (tuning records)
             if (const char *lp = std::getenv("EF_AUTOTUNE_LOG")) {
                 if (FILE *lf = std::fopen(lp, "a")) {
-                    std::fprintf(lf, "N=%d cells=%lld cluster=%d threads=%d variant=%d sg=%d paired=%d prefetch=%d ms=%.4f\n",
-                                 cp.N, (long long)n1, sh.cluster, sh.tpb, sh.occ, sh.sg_global, sh.paired, pfv, tmin);
+                    std::fprintf(lf, "N=%d cells=%lld cluster=%d threads=%d variant=%d sg=%d paired=%d prefetch=%d parts=%d ms=%.4f\n",
+                                 cp.N, (long long)n1, sh.cluster, sh.tpb, sh.occ, sh.sg_global, sh.paired, pfv, split, tmin);
                     std::fclose(lf);
                 }
             }
@@ -630,7 +795,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
         const Shape &sh = shapes[sweep[j].shape];
         double tmin = sweep[j].ms * (double)ncells_tune / (double)n1;
         if (ncells_tune > n1 && !sh.sg_global) {
-            e = time_one(sh, sweep[j].pf, ncells_tune, tmin);
+            e = time_one(sh, sweep[j].pf, sweep[j].split, ncells_tune, tmin);
             if (e != cudaSuccess) break;
             if (const char *lp = std::getenv("EF_AUTOTUNE_LOG")) {
                 if (FILE *lf = std::fopen(lp, "a")) {
@@ -645,6 +810,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
             best = tmin;
             best_sh = sh;
             best_pf = sweep[j].pf;
+            best_split = sweep[j].split;
         }
     }
     cudaFree(F);
@@ -652,14 +818,16 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune)
     cudaFree(sgws);
     cudaFree(fhws);
     cudaFree(dgws);
+    cudaFree(parts_ws);
     if (st) cudaStreamDestroy(st);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(e, "autotune");
     apply_shape(cp, best_sh);
     cp.prefetch = best_pf;
+    cp.split = best_split;
     cp.tuned_ms = best;
-    cache_store(key, best_sh.cluster, best_sh.tpb, best_sh.sg_global, best_pf, best_sh.paired, best_sh.occ, best);
+    cache_store(key, best_sh.cluster, best_sh.tpb, best_sh.sg_global, best_pf, best_sh.paired, best_sh.occ, best_split, best);
     return EF_OK;
 }
 
@@ -675,7 +843,7 @@ void *upload_table(const std::vector<double> &h, cudaError_t &err)
     return p;
 }
 
-ef_status build_class(const Desc &ds, ClassPlan &cp)
+ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split)
 {
     const int N = cp.N, d = ds.d;
     const int H = N / 2 + 1, N1 = d == 3 ? N : 1, NP = N1 * H;
@@ -791,7 +959,7 @@ ef_status build_class(const Desc &ds, ClassPlan &cp)
         if (e != cudaSuccess) return cuda_fail(e, "feature table");
         cp.nfeat = (int)modes.size() / 3;
     }
-    return choose_shape(ds, cp, cp.ncells > 0 ? std::min<int64_t>(cp.ncells, 2048) : 0);
+    return choose_shape(ds, cp, cp.ncells > 0 ? std::min<int64_t>(cp.ncells, 2048) : 0, may_split);
 }
 
 // Workspaces of one class for every cluster that can be resident at once (max_clusters, fixed by
@@ -799,26 +967,43 @@ ef_status build_class(const Desc &ds, ClassPlan &cp)
 // S/G slots.  Called once at plan creation, so that no operation allocates.
 ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
 {
-    const int slots_c = std::max(1, cp.max_clusters);
-    cudaError_t e = cudaMalloc(&cp.d_fh, (size_t)slots_c * ef::collide_fh_bytes(p->desc.prec, p->desc.d, cp.N));
+    const Desc &ds = p->desc;
+    const size_t el = ds.prec == EF_PREC_F32 ? 4 : 8;
+    const int64_t cell = (int64_t)cp.N * cp.N * (ds.d == 3 ? cp.N : 1);
+    std::vector<Shape> used(1, cp.cur);
+    if (!p->batched) used.insert(used.end(), cp.shapes.begin(), cp.shapes.end());
+    int64_t clusters = 1, sg_clusters = 0, part_cells = 0;
+    for (const Shape &sh : used) {
+        clusters = std::max<int64_t>(clusters, sh.max_clusters);
+        if (sh.sg_global) sg_clusters = std::max<int64_t>(sg_clusters, sh.max_clusters);
+        // uniform: n cells in S parts, n S at most the resident clusters, and nu: n (S + 1) <= 3/2 of them
+        if (!p->batched && max_split(ds, cp, sh, 1) > 1) part_cells = std::max<int64_t>(part_cells, sh.max_clusters + (sh.max_clusters + 1) / 2);
+    }
+    if (p->batched && cp.split > 1) part_cells = cp.ncells * (cp.split + 1);
+    cudaError_t e = cudaMalloc(&cp.d_fh, (size_t)clusters * ef::collide_fh_bytes(ds.prec, ds.d, cp.N));
     if (e != cudaSuccess) { cp.d_fh = nullptr; return cuda_fail(e, "spectrum workspace"); }
-    cp.fh_slots = slots_c;
-    if (!cp.sg_global) return EF_OK;
-    const int N = cp.N, N1 = p->desc.d == 3 ? N : 1;
-    const int64_t rows = (int64_t)cp.planes * N1;
-    const int64_t slots = (int64_t)slots_c * cp.cluster;
-    const size_t el = p->desc.prec == EF_PREC_F32 ? 4 : 8;
-    e = cudaMalloc(&cp.d_sg, (size_t)slots * 2 * rows * N * el);
-    if (e != cudaSuccess) { cp.d_sg = nullptr; return cuda_fail(e, "S/G workspace"); }
-    cp.sg_slots = slots;
+    cp.fh_slots = clusters;
+    if (sg_clusters) {
+        e = cudaMalloc(&cp.d_sg, (size_t)sg_clusters * 2 * cell * el);
+        if (e != cudaSuccess) { cp.d_sg = nullptr; return cuda_fail(e, "S/G workspace"); }
+        cp.sg_slots = sg_clusters;
+    }
+    if (part_cells) {
+        cp.part_bytes = (size_t)part_cells * cell * el;
+        cp.part_bytes = (cp.part_bytes + 255) / 256 * 256;
+        e = cudaMalloc(&cp.d_part, kPartSlots * cp.part_bytes);
+        if (e != cudaSuccess) { cp.d_part = nullptr; return cuda_fail(e, "part workspace"); }
+    }
     return EF_OK;
 }
 
-// The launch of grid_clusters clusters fits the workspaces made at plan creation (always true,
-// since the grid never exceeds max_clusters; checked so that a violation fails loudly).
-ef_status check_workspaces(const ClassPlan &cp, int grid_clusters)
+// The launch fits the workspaces made at plan creation (always true, since the grid never exceeds
+// max_clusters; checked so that a violation fails loudly).
+ef_status check_workspaces(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64_t n, int S, int grid_clusters)
 {
-    if (grid_clusters > cp.fh_slots || (cp.sg_global && (int64_t)grid_clusters * cp.cluster > cp.sg_slots))
+    const size_t cell = (size_t)cp.N * cp.N * (ds.d == 3 ? cp.N : 1) * (ds.prec == EF_PREC_F32 ? 4 : 8);
+    if (grid_clusters > cp.fh_slots || (sh.sg_global && grid_clusters > cp.sg_slots) ||
+        (S > 1 && (size_t)n * (S + 1) * cell > cp.part_bytes))
         return fail(EF_ERR_INVALID_ARG, "launch exceeds the plan's workspaces");
     return EF_OK;
 }
@@ -835,7 +1020,9 @@ void destroy_plan(ef_plan_s *p)
         cudaFree(cp.d_cell_id);
         cudaFree(cp.d_sg);
         cudaFree(cp.d_fh);
+        cudaFree(cp.d_part);
     }
+    if (p->split_done) cudaEventDestroy(p->split_done);
     cudaFree(p->d_all_off);
     cudaFree(p->d_all_N);
     cudaFree(p->d_rk);
@@ -905,11 +1092,97 @@ ef_status check_device(const ef_plan_s *p)
     return EF_OK;
 }
 
+// The shape and parts of a launch of n cells of one class.
+const Shape &call_shape(ef_plan_s *p, ClassPlan &cp, int64_t n, bool split, int &S)
+{
+    S = 1;
+    if (p->batched) {
+        if (split) S = cp.split;
+        return cp.cur;
+    }
+    pick_shape(p->desc, cp, n, p->sms);
+    if (split) S = cp.pick_s;
+    return cp.shapes[cp.pick_i];
+}
+
+// The part workspace of one operation: slot >= 0, or -1 where its calls are not split.  Calls share
+// workspace 0: each waits for an event behind the last one, whatever stream that was on.  (No
+// cudaStreamGetId: it ends a capture that is under way.)
+struct SplitUse {
+    ef_plan_s *p;
+    cudaStream_t s;
+    int slot = -1;
+    SplitUse(ef_plan_s *p_, int64_t ncells, cudaStream_t s_) : p(p_), s(s_)
+    {
+        bool wants = false;
+        for (ClassPlan &cp : p->classes) {
+            int S = 1;
+            const int64_t n = p->batched ? cp.ncells : ncells;
+            if (n > 0) call_shape(p, cp, n, true, S);
+            wants = wants || S > 1;
+        }
+        if (!wants) return;
+        if (!begin()) cudaGetLastError();
+    }
+    bool begin()
+    {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        unsigned long long capture = 0;
+        cudaGraph_t graph = nullptr;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
+        if (cap == cudaStreamCaptureStatusNone) {
+            if (p->split_used && cudaStreamWaitEvent(s, p->split_done, 0) != cudaSuccess) return false;
+            slot = 0;
+            return true;
+        }
+        if (cap != cudaStreamCaptureStatusActive || capture_info(s, &cap, &capture, &graph) != cudaSuccess) return false;
+        PartSlots &ps = *p->slots;
+        for (int i = 1; i < kPartSlots; ++i)
+            if (ps.taken[i].load() && ps.capture[i] == capture && ps.stream[i] == s) {
+                slot = i;
+                return true;
+            }
+        for (int i = 1; i < kPartSlots; ++i) {
+            int free_ = 0;
+            if (!ps.taken[i].compare_exchange_strong(free_, 1)) continue;
+            PartLease *l = new PartLease{p->slots, i};
+            cudaUserObject_t obj = nullptr;
+            if (cudaUserObjectCreate(&obj, l, end_lease, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+                end_lease(l);
+                return false;
+            }
+            if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+                cudaUserObjectRelease(obj, 1);            // runs end_lease
+                return false;
+            }
+            ps.capture[i] = capture;
+            ps.stream[i] = s;
+            slot = i;
+            return true;
+        }
+        return false;
+    }
+    static cudaError_t capture_info(cudaStream_t s, cudaStreamCaptureStatus *cap, unsigned long long *id, cudaGraph_t *graph)
+    {
+#if CUDART_VERSION >= 13000
+        return cudaStreamGetCaptureInfo(s, cap, id, graph, nullptr, nullptr, nullptr);
+#else
+        return cudaStreamGetCaptureInfo_v2(s, cap, id, graph, nullptr, nullptr);
+#endif
+    }
+    ~SplitUse()
+    {
+        if (slot != 0) return;
+        cudaEventRecord(p->split_done, s);
+        p->split_used = true;
+    }
+};
+
 // Enqueue one step: every size class on its own internal stream (forked from and joined back
 // to the caller's stream), each with a dynamic cell queue, so that clusters of one class fill
 // the SMs another class leaves idle.  A single class launches directly on the caller's stream.
 ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, double dt, double *diag,
-              cudaStream_t s)
+              int slot, cudaStream_t s)
 {
     const Desc &ds = p->desc;
     // size classes run back to back on the caller's stream unless EF_CONCURRENT_CLASSES=1 forks
@@ -929,8 +1202,10 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         ClassPlan &cp = p->classes[ci];
         const int64_t n = p->batched ? cp.ncells : ncells;
         if (n <= 0) continue;
-        const int grid = (int)std::min<int64_t>(n, cp.max_clusters);
-        ef_status st = check_workspaces(cp, grid);
+        int S = 1;
+        const Shape &sh = call_shape(p, cp, n, slot >= 0, S);
+        const int grid = (int)std::min<int64_t>(n * S, sh.max_clusters);
+        ef_status st = check_workspaces(ds, cp, sh, n, S, grid);
         if (st != EF_OK) return st;
         cudaStream_t cs = s;
         if (multi) {
@@ -947,14 +1222,16 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         a.cell_id = cp.d_cell_id;
         a.ncells = n;
         a.mult = cp.d_mult;
-        a.ops = cp.d_ops;
-        a.nops = cp.nops;
-        a.cluster = cp.cluster;
-        a.planes = cp.planes;
-        a.sg_global = cp.sg_global;
+        a.ops = sh.paired ? cp.d_ops_paired : cp.d_ops_single;
+        a.nops = sh.paired ? cp.nops_paired : cp.nops_single;
+        a.cluster = sh.cluster;
+        a.planes = sh.planes;
+        a.sg_global = sh.sg_global;
         a.sg_ws = cp.d_sg;
+        a.nsplit = S;
+        a.part = static_cast<unsigned char *>(cp.d_part) + (slot > 0 ? slot : 0) * cp.part_bytes;
         a.fh_ws = cp.d_fh;
-        a.npc = ef::collide_npc_v(ds.d, cp.N, cp.cluster, cp.occ);
+        a.npc = ef::collide_npc_v(ds.prec, ds.d, cp.N, sh.cluster, sh.occ);
         a.out_mode = mode;
         a.dt = dt;
         a.h = 2.0 * ds.L / cp.N;
@@ -962,8 +1239,8 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         a.status = p->d_status;
         a.counter = multi ? p->d_counters + ci : nullptr;
         a.prefetch = cp.prefetch;
-        a.paired = cp.paired;
-        e = launch_for(ds.prec, ds.d, cp.N, a, grid, cp.tpb, cp.smem, cp.occ, cs);
+        a.paired = sh.paired;
+        e = launch_shape(ds, cp.N, a, grid, sh, cs);
         if (e != cudaSuccess) return cuda_fail(e, "collide launch");
         if (multi) {
             e = cudaEventRecord(p->cevents[ci], cs);
@@ -978,10 +1255,15 @@ ef_status finish_plan(ef_plan_s *p)
 {
     cudaError_t e = cudaMalloc((void **)&p->d_status, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "status word");
+    e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
+    p->slots = std::make_shared<PartSlots>();
+    if (e == cudaSuccess) e = ef::split_finish_setup(p->desc.prec == EF_PREC_F32 ? 0 : 1, p->desc.d);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->split_done, cudaEventDisableTiming);
+    if (e != cudaSuccess) return cuda_fail(e, "plan event");
     e = cudaMemset(p->d_status, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "status word");
     for (ClassPlan &cp : p->classes) {
-        ef_status st = build_class(p->desc, cp);
+        ef_status st = build_class(p->desc, cp, p->may_split);
         if (st != EF_OK) return st;
         st = alloc_workspaces(p, cp);
         if (st != EF_OK) return st;
@@ -1100,6 +1382,16 @@ ef_status ef_plan_create(int d, int N, double L, ef_kernel kernel, int R, ef_pre
 ef_status ef_plan_create_batched(int d, int64_t ncells, const int *N_host, double L, ef_kernel kernel, int R,
                                  ef_precision prec, ef_plan_t *out)
 {
+    return ef::ef_plan_create_batched_opt(d, ncells, N_host, L, kernel, R, prec, true, out);
+}
+
+}  // extern "C"
+
+namespace ef {
+
+ef_status ef_plan_create_batched_opt(int d, int64_t ncells, const int *N_host, double L, ef_kernel kernel, int R, ef_precision prec,
+                              bool may_split, ef_plan_t *out)
+{
     if (!out) return fail(EF_ERR_INVALID_ARG, "null output handle");
     *out = nullptr;
     if (ncells <= 0 || !N_host) return fail(EF_ERR_INVALID_ARG, "batched plan needs ncells > 0 and N_host");
@@ -1129,6 +1421,7 @@ ef_status ef_plan_create_batched(int d, int64_t ncells, const int *N_host, doubl
     ef_plan_s *p = new ef_plan_s();
     p->desc = ds;
     p->batched = true;
+    p->may_split = may_split;
     p->ncells = ncells;
     cudaError_t e = cudaGetDevice(&p->device);
     if (e != cudaSuccess) { delete p; return cuda_fail(e, "cudaGetDevice"); }
@@ -1160,6 +1453,10 @@ ef_status ef_plan_create_batched(int d, int64_t ncells, const int *N_host, doubl
     return EF_OK;
 }
 
+}  // namespace ef
+
+extern "C" {
+
 ef_status ef_plan_destroy(ef_plan_t plan)
 {
     if (!plan) return fail(EF_ERR_INVALID_ARG, "null plan");
@@ -1172,17 +1469,18 @@ ef_status ef_plan_destroy(ef_plan_t plan)
 namespace {
 
 // One step (all size classes) either launched directly or through the plan's cached CUDA graph.
-ef_status step(ef_plan_s *p, const void *F, void *Q, int64_t ncells, int mode, double dt, double *diag, cudaStream_t s)
+ef_status step(ef_plan_s *p, const void *F, void *Q, int64_t ncells, int mode, double dt, double *diag, int slot,
+               cudaStream_t s)
 {
-    if (!(p->use_graph && s != nullptr)) return run(p, F, Q, ncells, mode, dt, diag, s);
+    if (!(p->use_graph && s != nullptr)) return run(p, F, Q, ncells, mode, dt, diag, slot, s);
     const bool hit = p->gexec && p->g_F == F && p->g_Q == Q && p->g_n == ncells && p->g_stream == s &&
-                     p->g_mode == mode && p->g_dt == dt && p->g_diag == diag;
+                     p->g_mode == mode && p->g_dt == dt && p->g_diag == diag && p->g_slot == slot;
     if (!hit) {
         if (p->gexec) { cudaGraphExecDestroy(p->gexec); p->gexec = nullptr; }
         ef_status st;
         cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
-        st = run(p, F, Q, ncells, mode, dt, diag, s);
+        st = run(p, F, Q, ncells, mode, dt, diag, slot, s);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(s, &g);
         if (st != EF_OK) { if (g) cudaGraphDestroy(g); return st; }
@@ -1197,6 +1495,7 @@ ef_status step(ef_plan_s *p, const void *F, void *Q, int64_t ncells, int mode, d
         p->g_mode = mode;
         p->g_dt = dt;
         p->g_diag = diag;
+        p->g_slot = slot;
     }
     cudaError_t e = cudaGraphLaunch(p->gexec, s);
     if (e != cudaSuccess) return cuda_fail(e, "graph launch");
@@ -1286,7 +1585,8 @@ ef_status ef_collide(ef_plan_t p, const void *F, void *Q, int64_t ncells, ef_str
     if (((uintptr_t)F | (uintptr_t)Q) % 16) return fail(EF_ERR_INVALID_ARG, "F and Q must be 16-byte aligned");
     ef_status st = check_device(p);
     if (st != EF_OK) return st;
-    return step(p, F, Q, ncells, ef::OUT_COLLIDE, 0.0, nullptr, (cudaStream_t)stream);
+    const SplitUse use(p, ncells, (cudaStream_t)stream);
+    return step(p, F, Q, ncells, ef::OUT_COLLIDE, 0.0, nullptr, use.slot, (cudaStream_t)stream);
 }
 
 ef_status ef_euler_step(ef_plan_t p, void *F, double dt, int nsteps, double *diag, int64_t ncells, ef_stream_t stream)
@@ -1300,9 +1600,10 @@ ef_status ef_euler_step(ef_plan_t p, void *F, double dt, int nsteps, double *dia
     if ((uintptr_t)F % 16) return fail(EF_ERR_INVALID_ARG, "F must be 16-byte aligned");
     ef_status st = check_device(p);
     if (st != EF_OK) return st;
+    const SplitUse use(p, ncells, (cudaStream_t)stream);
     for (int k = 0; k < nsteps; ++k) {
         st = step(p, F, F, ncells, ef::OUT_EULER, dt, diag ? diag + (int64_t)k * ncells * ef::kDiag : nullptr,
-                  (cudaStream_t)stream);
+                  use.slot, (cudaStream_t)stream);
         if (st != EF_OK) return st;
     }
     return EF_OK;
@@ -1371,18 +1672,19 @@ ef_status ef_rk3_step(ef_plan_t p, void *F, double dt, int nsteps, double *diag,
     void *A = p->d_rk, *B = static_cast<unsigned char *>(p->d_rk) + half;
     cudaStream_t s = (cudaStream_t)stream;
     const int prec = ds.prec == EF_PREC_F32 ? 0 : 1;
+    const SplitUse use(p, ncells, s);
     for (int k = 0; k < nsteps; ++k) {
         double *dk = diag ? diag + (int64_t)k * ncells * ef::kDiag : nullptr;
         // F1 = F + dt Q[F]
-        st = run(p, F, A, ncells, ef::OUT_EULER, dt, dk, s);
+        st = run(p, F, A, ncells, ef::OUT_EULER, dt, dk, use.slot, s);
         if (st != EF_OK) return st;
         // F2 = 3/4 F + 1/4 (F1 + dt Q[F1])
-        st = run(p, A, B, ncells, ef::OUT_EULER, dt, nullptr, s);
+        st = run(p, A, B, ncells, ef::OUT_EULER, dt, nullptr, use.slot, s);
         if (st != EF_OK) return st;
         cudaError_t e = ef::axpby_launch(prec, B, F, B, 0.75, 0.25, total, s);
         if (e != cudaSuccess) return cuda_fail(e, "RK3 combine");
         // F <- 1/3 F + 2/3 (F2 + dt Q[F2])
-        st = run(p, B, A, ncells, ef::OUT_EULER, dt, nullptr, s);
+        st = run(p, B, A, ncells, ef::OUT_EULER, dt, nullptr, use.slot, s);
         if (st != EF_OK) return st;
         e = ef::axpby_launch(prec, F, F, A, 1.0 / 3.0, 2.0 / 3.0, total, s);
         if (e != cudaSuccess) return cuda_fail(e, "RK3 combine");

@@ -123,7 +123,8 @@ ef_status ef_stream_plan_create(int d, int64_t ncells, const int *N_host, double
         }
         ch.nc = c - ch.c0;
         ch.ne = elem - ch.e0;
-        ef_status st = ef_plan_create_batched(d, ch.nc, N_host + ch.c0, L, kernel, R, prec, &ch.plan);
+        // chunks share the device: parts would repeat forward transforms on SMs that other chunks fill
+        ef_status st = ef::ef_plan_create_batched_opt(d, ch.nc, N_host + ch.c0, L, kernel, R, prec, false, &ch.plan);
         if (st != EF_OK) { sp_free(sp); return st; }
         if ((int)sp->comp.size() < kComputeStreams) {
             cudaStream_t q = nullptr;
