@@ -1,5 +1,4 @@
-// Collide kernel instantiations: double, 2D.
-#define EF_T double
+// FP64 collide kernel instantiations, 2D.
 #define EF_D 2
 #define EF_SUF f64_2d
-#include "ef_collide_variant.inc"
+#include "ef_collide_q_variant.inc"

@@ -103,6 +103,7 @@ inline int collide_npc_v(int prec, int d, int N, int C, int occ)
         const int np = N * N / 2;
         return (np % C == 0 && (np / C) % 2 == 0) ? np / C : 0;
     }
+    if (prec == 1) return ((d == 3 ? N : 1) * (N / 2) + C - 1) / C;
     return collide_npc(d, N, C);
 }
 cudaError_t collide_launch(int prec, int d, int N, const CollideArgs &a, int grid_clusters, int tpb, size_t smem,

@@ -450,7 +450,7 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
                 if (rows % 2) continue;
                 const int nb = paired ? 2 : 1;
                 // FP64: four lanes per line, N/2 stored columns (ef_collide_q.cuh)
-                const bool quad = false;
+                const bool quad = ds.prec == EF_PREC_F64;
                 const int need = quad ? 4 * std::max({nb * ef::collide_npc_v(1, d, N, C, 1), paired ? rows : rows / 2,
                                                       d == 3 ? nb * planes * (N / 2) : 1})
                                       : std::max({nb * ef::collide_npc(d, N, C), paired ? rows : rows / 2,
