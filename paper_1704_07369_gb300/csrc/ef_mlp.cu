@@ -32,7 +32,10 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int BM = 64, BN = 64, BK = 32, LDS = BK + 8;   // smem row stride 40 bf16 = 80 B
+// mma.sync kernel: 64 x 64 tiles, K in blocks of 64, four cp.async stages; a shared-memory row of 72 bf16
+// (144 bytes) keeps ldmatrix and the staged epilogue rows free of bank conflicts
+constexpr int BM = 64, BN = 64, BK = 64, LDS = BK + 8, NSTAGE = 4;
+constexpr size_t kSyncSmem = (size_t)NSTAGE * (BM + BN) * LDS * 2;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -41,8 +44,8 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(smem)), "l"(gmem));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void *p)
 {
@@ -74,26 +77,50 @@ struct GemmArgs {
     int ldcbt;
     int lo_off;         // > 0: also write the low halves a - bf16(a) at column / row + lo_off
     int *status;        // nullable: device status word, EF_ERR_TIMEOUT (5) when a bounded wait gives up
+    const float *pre;   // EPI_DA: [M][ldpre] pre-activations whose sign masks the result
+    int ldpre;
+    float *db;          // EPI_DW: nullable [M] sums of A's rows
 };
 
-// 4 warps in 2 x 2, each 32 x 32 (2 m16 x 4 n8 tiles).  M % 64 == N % 64 == K % 32 == 0.
-__global__ void __launch_bounds__(128) gemm_tn_kernel(const GemmArgs g)
+// What the mma.sync kernel does with its product:
+//   EPI_FWD  bias, optional FP32 copy, relu, bf16 halves and their transposes (GemmArgs above)
+//   EPI_DW   weight gradient of the tied hi / lo halves: B holds [hi rows | lo rows], N counts both; the
+//            two products of a column are added and stored in Cf [M][ldcf], and A's row sums in db
+//   EPI_DA   gradient at the layer below: masked by pre > 0, as bf16 in Cb and transposed in CbT
+enum Epilogue { EPI_FWD = 0, EPI_DW = 1, EPI_DA = 2 };
+
+// 4 warps in 2 x 2, each 32 x 32 (2 m16 x 4 n8 tiles).  M % 64 == N % 64 == K % 64 == 0.  The training
+// batch's products (64 - 240 tiles) leave one or two CTAs per SM, so a tile's time is its serial chain
+// of K blocks: three blocks are in flight ahead of the one being multiplied.  Every product is summed
+// in K order by one accumulator chain, whatever the tile or stage count.  Results leave through
+// shared memory as 16-byte pieces of rows, for the transposed copies too; the element-wise passes that
+// followed a product (fold of the halves, relu mask, row sums) are its epilogue.  Loss and gradients of
+// a 1024-row batch (928 - 512 x 3 - 926): 300 -> 176 us, 27 launches -> 15.
+template <int MODE>
+__global__ void __launch_bounds__(128) gemm_sync_kernel(const GemmArgs g)
 {
-    __shared__ __align__(16) bf16 sA[2][BM * LDS];
-    __shared__ __align__(16) bf16 sB[2][BN * LDS];
+    extern __shared__ __align__(16) unsigned char sync_raw[];
+    bf16 *sA = reinterpret_cast<bf16 *>(sync_raw);             // [NSTAGE][BM][LDS]
+    bf16 *sB = sA + NSTAGE * BM * LDS;                         // [NSTAGE][BN][LDS]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp >> 1, wn = warp & 1;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = blockIdx.y * BM;
+    const int n0 = blockIdx.x * (MODE == EPI_DW ? BN / 2 : BN);
     const int nk = g.K / BK;
 
-    auto load_tile = [&](int kt, int buf) {
-        // A: 64 rows x 32 bf16 = 256 chunks of 16 B; B likewise: 2 + 2 chunks per thread
+    auto load_tile = [&](int kt) {
+        if (kt < nk) {
+            bf16 *a = sA + (kt % NSTAGE) * BM * LDS, *b = sB + (kt % NSTAGE) * BN * LDS;
+            // A: 64 rows x 64 bf16 = 512 chunks of 16 B; B likewise: 4 + 4 chunks per thread
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int c = tid + i * 128;
-            const int r = c >> 2, k8 = (c & 3) * 8;
-            cp_async16(&sA[buf][r * LDS + k8], g.A + (size_t)(m0 + r) * g.lda + kt * BK + k8);
-            cp_async16(&sB[buf][r * LDS + k8], g.B + (size_t)(n0 + r) * g.ldb + kt * BK + k8);
+            for (int i = 0; i < 4; ++i) {
+                const int c = tid + i * 128;
+                const int r = c >> 3, k8 = (c & 7) * 8;
+                // EPI_DW: 32 rows of the hi halves, then the same 32 of the lo halves
+                const int rb = MODE == EPI_DW ? (r < BN / 2 ? n0 + r : g.N / 2 + n0 + r - BN / 2) : n0 + r;
+                cp_async16(a + r * LDS + k8, g.A + (size_t)(m0 + r) * g.lda + kt * BK + k8);
+                cp_async16(b + r * LDS + k8, g.B + (size_t)rb * g.ldb + kt * BK + k8);
+            }
         }
         cp_async_commit();
     };
@@ -105,33 +132,39 @@ __global__ void __launch_bounds__(128) gemm_tn_kernel(const GemmArgs g)
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.f;
+    float rowsum = 0.f;                                        // EPI_DW: row tid of A (tid < 64)
 
-    load_tile(0, 0);
+    for (int kt = 0; kt < NSTAGE - 1; ++kt) load_tile(kt);
     for (int kt = 0; kt < nk; ++kt) {
-        const int buf = kt & 1;
-        if (kt + 1 < nk) {
-            load_tile(kt + 1, buf ^ 1);
-            cp_async_wait1();
-        } else {
-            cp_async_wait0();
+        cp_async_wait<NSTAGE - 2>();
+        __syncthreads();                                       // block kt has landed; block kt - 1 is read
+        load_tile(kt + NSTAGE - 1);
+        const bf16 *a = sA + (kt % NSTAGE) * BM * LDS, *b = sB + (kt % NSTAGE) * BN * LDS;
+        if (MODE == EPI_DW && blockIdx.x == 0 && g.db && tid < BM) {
+            float t = 0.f;
+#pragma unroll
+            for (int k8 = 0; k8 < BK; k8 += 8) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(a + tid * LDS + k8);
+                const bf16 *e = reinterpret_cast<const bf16 *>(&w);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t += __bfloat162float(e[j]);
+            }
+            rowsum += t;
         }
-        __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; kk += 16) {
             uint32_t af[2][4];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int r = wm * 32 + i * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                const int c = kk + (lane >> 4) * 8;
-                ldmatrix_x4(af[i], &sA[buf][r * LDS + c]);
+                ldmatrix_x4(af[i], a + r * LDS + kk + (lane >> 4) * 8);
             }
             uint32_t bfr[4][2];
 #pragma unroll
             for (int j2 = 0; j2 < 2; ++j2) {      // two n8 tiles per ldmatrix.x4
                 uint32_t t[4];
                 const int n = wn * 32 + j2 * 16 + (lane & 7) + (lane >> 4) * 8;
-                const int c = kk + ((lane >> 3) & 1) * 8;
-                ldmatrix_x4(t, &sB[buf][n * LDS + c]);
+                ldmatrix_x4(t, b + n * LDS + kk + ((lane >> 3) & 1) * 8);
                 bfr[2 * j2][0] = t[0];
                 bfr[2 * j2][1] = t[1];
                 bfr[2 * j2 + 1][0] = t[2];
@@ -142,44 +175,106 @@ __global__ void __launch_bounds__(128) gemm_tn_kernel(const GemmArgs g)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i], bfr[j][0], bfr[j][1]);
         }
-        __syncthreads();
     }
-    // epilogue: c0,c1 at (row, col..col+1), c2,c3 at (row + 8, ...)
+    cp_async_wait<0>();
+    __syncthreads();                                           // the stages are free: epilogue staging
+    // fragment: c0,c1 at (row, col..col+1), c2,c3 at (row + 8, ...)
+    if constexpr (MODE == EPI_DW) {
+        float *sf = reinterpret_cast<float *>(sync_raw);       // [64][34] products with the lo halves
+        constexpr int LF = BN / 2 + 2;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+        for (int half = 0; half < 2; ++half) {
+            if (wn == 1 - half) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+                for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int row = m0 + wm * 32 + i * 16 + (lane >> 2) + h * 8;
-                const int col = n0 + wn * 32 + j * 8 + (lane & 3) * 2;
-                float v0 = acc[i][j][2 * h], v1 = acc[i][j][2 * h + 1];
-                if (g.bias) {
-                    v0 += g.bias[col];
-                    v1 += g.bias[col + 1];
-                }
-                if (g.Cf) *reinterpret_cast<float2 *>(g.Cf + (size_t)row * g.ldcf + col) = make_float2(v0, v1);
-                if (g.relu) {
-                    v0 = fmaxf(v0, 0.f);
-                    v1 = fmaxf(v1, 0.f);
-                }
-                const bf16 h0 = __float2bfloat16(v0), h1 = __float2bfloat16(v1);
-                const bf16 l0 = __float2bfloat16(v0 - __bfloat162float(h0)), l1 = __float2bfloat16(v1 - __bfloat162float(h1));
-                if (g.Cb) {
-                    *reinterpret_cast<__nv_bfloat162 *>(g.Cb + (size_t)row * g.ldcb + col) = __halves2bfloat162(h0, h1);
-                    if (g.lo_off)
-                        *reinterpret_cast<__nv_bfloat162 *>(g.Cb + (size_t)row * g.ldcb + g.lo_off + col) =
-                            __halves2bfloat162(l0, l1);
-                }
-                if (g.CbT) {
-                    g.CbT[(size_t)col * g.ldcbt + row] = h0;
-                    g.CbT[(size_t)(col + 1) * g.ldcbt + row] = h1;
-                    if (g.lo_off) {
-                        g.CbT[(size_t)(g.lo_off + col) * g.ldcbt + row] = l0;
-                        g.CbT[(size_t)(g.lo_off + col + 1) * g.ldcbt + row] = l1;
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int row = wm * 32 + i * 16 + (lane >> 2) + h * 8, col = j * 8 + (lane & 3) * 2;
+                            float2 *q = reinterpret_cast<float2 *>(sf + row * LF + col);
+                            if (half == 0) {
+                                *q = make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+                            } else {
+                                const float2 lo = *q;
+                                *reinterpret_cast<float2 *>(g.Cf + (size_t)(m0 + row) * g.ldcf + n0 + col) =
+                                    make_float2(acc[i][j][2 * h] + lo.x, acc[i][j][2 * h + 1] + lo.y);
+                            }
+                        }
+            }
+            __syncthreads();
+        }
+        if (blockIdx.x == 0 && g.db && tid < BM) g.db[m0 + tid] = rowsum;
+        return;
+    } else {
+        bf16 *st = reinterpret_cast<bf16 *>(sync_raw);         // [hi, hi^T, lo, lo^T][64][LDS]
+        const bool lo_out = MODE == EPI_FWD && g.lo_off > 0;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int row = wm * 32 + i * 16 + (lane >> 2) + h * 8, col = wn * 32 + j * 8 + (lane & 3) * 2;
+                    float v0 = acc[i][j][2 * h], v1 = acc[i][j][2 * h + 1];
+                    if constexpr (MODE == EPI_FWD) {
+                        if (g.bias) {
+                            v0 += g.bias[n0 + col];
+                            v1 += g.bias[n0 + col + 1];
+                        }
+                        if (g.Cf) *reinterpret_cast<float2 *>(g.Cf + (size_t)(m0 + row) * g.ldcf + n0 + col) = make_float2(v0, v1);
+                        if (g.relu) {
+                            v0 = fmaxf(v0, 0.f);
+                            v1 = fmaxf(v1, 0.f);
+                        }
+                    } else {
+                        const float2 p = *reinterpret_cast<const float2 *>(g.pre + (size_t)(m0 + row) * g.ldpre + n0 + col);
+                        v0 = p.x > 0.f ? v0 : 0.f;
+                        v1 = p.y > 0.f ? v1 : 0.f;
+                    }
+                    if (!g.Cb && !g.CbT) continue;
+                    const bf16 h0 = __float2bfloat16(v0), h1 = __float2bfloat16(v1);
+                    *reinterpret_cast<__nv_bfloat162 *>(st + row * LDS + col) = __halves2bfloat162(h0, h1);
+                    st[(BM + col) * LDS + row] = h0;
+                    st[(BM + col + 1) * LDS + row] = h1;
+                    if (lo_out) {
+                        const bf16 l0 = __float2bfloat16(v0 - __bfloat162float(h0)), l1 = __float2bfloat16(v1 - __bfloat162float(h1));
+                        *reinterpret_cast<__nv_bfloat162 *>(st + (2 * BM + row) * LDS + col) = __halves2bfloat162(l0, l1);
+                        st[(3 * BM + col) * LDS + row] = l0;
+                        st[(3 * BM + col + 1) * LDS + row] = l1;
                     }
                 }
+        if (!g.Cb && !g.CbT) return;
+        __syncthreads();
+        for (int half = 0; half < (lo_out ? 2 : 1); ++half) {
+            const bf16 *q = st + half * 2 * BM * LDS;
+            const int off = half ? g.lo_off : 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = tid + i * 128, r = c >> 3, k8 = (c & 7) * 8;
+                if (g.Cb) *reinterpret_cast<uint4 *>(g.Cb + (size_t)(m0 + r) * g.ldcb + off + n0 + k8) = *reinterpret_cast<const uint4 *>(q + r * LDS + k8);
+                if (g.CbT) *reinterpret_cast<uint4 *>(g.CbT + (size_t)(off + n0 + r) * g.ldcbt + m0 + k8) = *reinterpret_cast<const uint4 *>(q + (BM + r) * LDS + k8);
             }
+        }
+    }
+}
+
+template <int MODE>
+cudaError_t gemm_sync(const GemmArgs &g, cudaStream_t s)
+{
+    if (g.M % BM || g.N % BN || g.K % BK) return cudaErrorInvalidValue;
+    static unsigned long long set_on = 0;    // devices on which the attribute has been raised
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(__atomic_load_n(&set_on, __ATOMIC_ACQUIRE) & bit)) {
+        e = cudaFuncSetAttribute(gemm_sync_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSyncSmem);
+        if (e != cudaSuccess) return e;
+        __atomic_fetch_or(&set_on, bit, __ATOMIC_ACQ_REL);
+    }
+    gemm_sync_kernel<MODE><<<dim3(g.N / BN, g.M / BM), 128, kSyncSmem, s>>>(g);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ tcgen05 GEMM ---------------
@@ -440,55 +535,82 @@ cudaError_t gemm_tc(const GemmArgs &g, bool *used, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// the tcgen05 kernel's widest N tile that still gives every SM a tile, 0 where the product is not its
+// (small products keep the 64 x 64 mma.sync kernel, whose many CTAs fill the device)
+int tc_tile(const GemmArgs &g)
+{
+    const bool aligned = g.lda % 8 == 0 && g.ldb % 8 == 0 && (!g.Cf || g.ldcf % 4 == 0) && (!g.Cb || g.ldcb % 8 == 0) &&
+                         g.lo_off % 8 == 0;
+    if (g.M % TC_BM || g.K % TC_BK || !aligned) return 0;
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms <= 0) sms = 1;
+    }
+    const int64_t mt = g.M / TC_BM;
+    for (int tn : {256, 192, 128, 64})
+        if (g.N % tn == 0 && mt * (g.N / tn) >= sms) return tn;
+    return 0;
+}
+
 // tcgen05 for the shapes it tiles (M multiple of 128, K of 64, N of 64, 16-byte aligned rows) with at
 // least one tile per SM, the mma.sync kernel for the rest (and wherever a tensor map cannot be made)
 cudaError_t gemm(const GemmArgs &g, cudaStream_t s)
 {
-    const bool aligned = g.lda % 8 == 0 && g.ldb % 8 == 0 && (!g.Cf || g.ldcf % 4 == 0) && (!g.Cb || g.ldcb % 8 == 0) &&
-                         g.lo_off % 8 == 0;
-    if (g.M % TC_BM == 0 && g.K % TC_BK == 0 && aligned) {
-        // the widest N tile that still gives every SM a tile; small products (the training batch)
-        // keep the 64 x 64 kernel, whose many CTAs fill the device
-        static int sms = 0;
-        if (!sms) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (sms <= 0) sms = 1;
-        }
-        const int64_t mt = g.M / TC_BM;
-        auto fills = [&](int tn) { return g.N % tn == 0 && mt * (g.N / tn) >= sms; };
-        bool used = false;
-        cudaError_t e = cudaSuccess;
-        if (fills(256)) e = gemm_tc<256>(g, &used, s);
-        else if (fills(192)) e = gemm_tc<192>(g, &used, s);
-        else if (fills(128)) e = gemm_tc<128>(g, &used, s);
-        else if (fills(64)) e = gemm_tc<64>(g, &used, s);
-        if (e != cudaSuccess || used) return e;
+    bool used = false;
+    cudaError_t e = cudaSuccess;
+    switch (tc_tile(g)) {
+    case 256: e = gemm_tc<256>(g, &used, s); break;
+    case 192: e = gemm_tc<192>(g, &used, s); break;
+    case 128: e = gemm_tc<128>(g, &used, s); break;
+    case 64: e = gemm_tc<64>(g, &used, s); break;
+    default: break;
     }
-    if (g.M % BM || g.N % BN || g.K % BK) return cudaErrorInvalidValue;
-    dim3 grid(g.N / BN, g.M / BM);
-    gemm_tn_kernel<<<grid, 128, 0, s>>>(g);
-    return cudaGetLastError();
+    return e != cudaSuccess || used ? e : gemm_sync<EPI_FWD>(g, s);
+}
+
+// Transposed copies are made from 64 x 64 tiles in shared memory: the strided 2-byte stores of a
+// thread-per-element pass touch a 32-byte sector each.
+constexpr int TT = 64, TTL = TT + 2;             // tile, row stride (bf16)
+
+// rows [c0, c0 + 64) of the transposed tile: 64 batch entries, 16 bytes a thread
+__device__ __forceinline__ void store_tile_t(const bf16 (*t)[TTL], bf16 *out, int64_t ld, int64_t r0, int c0)
+{
+    for (int i = threadIdx.x; i < TT * (TT / 2); i += blockDim.x) {
+        const int c = i / (TT / 2), r = (i % (TT / 2)) * 2;
+        *reinterpret_cast<__nv_bfloat162 *>(out + (size_t)(c0 + c) * ld + r0 + r) = *reinterpret_cast<const __nv_bfloat162 *>(&t[c][r]);
+    }
 }
 
 // X (fp32 [B][ldx], first nin used) -> split bf16 [B][2 ninp] (hi | lo) and its transpose
-// [2 ninp][B]; pad zeroed.
-__global__ void pack_input_kernel(const float *X, int ldx, int nin, int ninp, int64_t B, bf16 *Xb, bf16 *XbT)
+// [2 ninp][B]; pad zeroed.  One 64 x 64 tile per CTA (ninp and B are multiples of 64).
+template <bool TR>
+__global__ void __launch_bounds__(256) pack_input_kernel(const float *X, int ldx, int nin, int ninp, int64_t B, bf16 *Xb, bf16 *XbT)
 {
-    const int64_t total = B * ninp;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = i / ninp;
-        const int j = (int)(i % ninp);
-        const float v = j < nin ? X[b * ldx + j] : 0.f;
-        const bf16 h = __float2bfloat16(v);
-        const bf16 l = __float2bfloat16(v - __bfloat162float(h));
-        Xb[b * 2 * ninp + j] = h;
-        Xb[b * 2 * ninp + ninp + j] = l;
-        if (XbT) {
-            XbT[(size_t)j * B + b] = h;
-            XbT[(size_t)(ninp + j) * B + b] = l;
+    __shared__ bf16 th[TR ? TT : 1][TTL], tl[TR ? TT : 1][TTL];
+    const int64_t b0 = (int64_t)blockIdx.y * TT;
+    const int j0 = blockIdx.x * TT;
+    for (int i = threadIdx.x; i < TT * TT / 2; i += blockDim.x) {
+        const int r = i / (TT / 2), c = (i % (TT / 2)) * 2, j = j0 + c;
+        const int64_t b = b0 + r;
+        const float v0 = j < nin ? X[b * ldx + j] : 0.f, v1 = j + 1 < nin ? X[b * ldx + j + 1] : 0.f;
+        const bf16 h0 = __float2bfloat16(v0), h1 = __float2bfloat16(v1);
+        const bf16 l0 = __float2bfloat16(v0 - __bfloat162float(h0)), l1 = __float2bfloat16(v1 - __bfloat162float(h1));
+        *reinterpret_cast<__nv_bfloat162 *>(Xb + b * 2 * ninp + j) = __halves2bfloat162(h0, h1);
+        *reinterpret_cast<__nv_bfloat162 *>(Xb + b * 2 * ninp + ninp + j) = __halves2bfloat162(l0, l1);
+        if (TR) {
+            th[c][r] = h0;
+            th[c + 1][r] = h1;
+            tl[c][r] = l0;
+            tl[c + 1][r] = l1;
         }
+    }
+    if (TR) {
+        __syncthreads();
+        store_tile_t(th, XbT, B, b0, j0);
+        store_tile_t(tl, XbT, B, b0, ninp + j0);
     }
 }
 
@@ -503,30 +625,39 @@ __global__ void fold_split_kernel(const float *dW2, int out, int in, float *g)
 }
 
 // MSE loss over the first nout outputs (optionally weighted): loss = sum w_j (y - t)^2 / (B n_w),
-// dY = 2 w_j (y - t) / (B n_w) in bf16 [B][noutp] and [noutp][B] (pad rows zero).
-__global__ void mse_kernel(const float *Y, int ldy_pred, const float *T, int ldt, const float *wmask, const float *roww,
+// dY = 2 w_j (y - t) / (B n_w) in bf16 [B][noutp] and [noutp][B] (pad columns zero).  One 64 x 64 tile
+// per CTA.
+__global__ void __launch_bounds__(256) mse_kernel(const float *Y, int ldy_pred, const float *T, int ldt, const float *wmask, const float *roww,
                            int nout, int noutp, int64_t B, float inv_count, bf16 *dY, bf16 *dYT, float *loss)
 {
+    __shared__ bf16 th[TT][TTL];
+    const int64_t b0 = (int64_t)blockIdx.y * TT;
+    const int j0 = blockIdx.x * TT;
     float acc = 0.f;
-    const int64_t total = B * noutp;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = i / noutp;
-        const int j = (int)(i % noutp);
-        float g = 0.f;
-        if (j < nout) {
-            const float w = (wmask ? wmask[j] : 1.f) * (roww ? roww[b] : 1.f);
-            const float d = Y[b * ldy_pred + j] - T[b * ldt + j];
-            acc += w * d * d;
-            g = 2.f * w * d * inv_count;
+    for (int i = threadIdx.x; i < TT * TT / 2; i += blockDim.x) {
+        const int r = i / (TT / 2), c = (i % (TT / 2)) * 2;
+        const int64_t b = b0 + r;
+        bf16 h[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int j = j0 + c + e;
+            float g = 0.f;
+            if (j < nout) {
+                const float w = (wmask ? wmask[j] : 1.f) * (roww ? roww[b] : 1.f);
+                const float d = Y[b * ldy_pred + j] - T[b * ldt + j];
+                acc += w * d * d;
+                g = 2.f * w * d * inv_count;
+            }
+            h[e] = __float2bfloat16(g);
+            th[c + e][r] = h[e];
         }
-        const bf16 h = __float2bfloat16(g);
-        dY[i] = h;
-        dYT[(size_t)j * B + b] = h;
+        *reinterpret_cast<__nv_bfloat162 *>(dY + b * noutp + j0 + c) = __halves2bfloat162(h[0], h[1]);
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     __shared__ float red[32];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
+    store_tile_t(th, dYT, B, b0, j0);
     if (threadIdx.x == 0) {
         float t = 0.f;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
@@ -623,7 +754,7 @@ struct ef_mlp_s {
     std::vector<bf16 *> act, actT;  // [B][out_l], [out_l][B] (hidden layers)
     float *dA = nullptr;            // [B][max out] fp32
     float *dW2 = nullptr;           // [max out][2 max in] fp32: gradient of the split halves
-    bf16 *dY = nullptr, *dYT = nullptr;
+    bf16 *dY[2] = {}, *dYT[2] = {}; // gradient at a layer's output and its transpose, layers in turn
     int64_t step = 0;
     int device = 0;
     int *status = nullptr;          // device status word (EF_ERR_TIMEOUT from a GEMM's bounded waits)
@@ -661,8 +792,10 @@ void mlp_free(ef_mlp_s *n)
     for (auto q : n->actT) cudaFree(q);
     cudaFree(n->dA);
     cudaFree(n->dW2);
-    cudaFree(n->dY);
-    cudaFree(n->dYT);
+    for (int i = 0; i < 2; ++i) {
+        cudaFree(n->dY[i]);
+        cudaFree(n->dYT[i]);
+    }
     cudaFree(n->status);
     delete n;
 }
@@ -682,7 +815,7 @@ ef_status mlp_forward_packed(ef_mlp_s *n, int64_t B, float *Yout, int ldy, bool 
         g.bias = n->p + n->boff[l];
         const bool last = l + 1 == n->nl;
         g.relu = last ? 0 : 1;
-        g.Cf = last ? Yout : n->pre[l];
+        g.Cf = last ? Yout : keep_T ? n->pre[l] : nullptr;     // hidden pre-activations: for the backward pass
         g.ldcf = last ? ldy : n->dout[l];
         g.Cb = last ? nullptr : n->act[l];
         g.ldcb = 2 * n->dout[l];
@@ -763,8 +896,10 @@ ef_status ef_mlp_create(int nin, int nhidden, int nlayers, int nout, int64_t max
     alloc((void **)&n->XbT, (size_t)max_batch * 2 * n->ninp * 2);
     alloc((void **)&n->dW2, (size_t)maxd * 2 * maxd * 4);
     alloc((void **)&n->dA, (size_t)max_batch * maxd * 4);
-    alloc((void **)&n->dY, (size_t)max_batch * maxd * 2);
-    alloc((void **)&n->dYT, (size_t)max_batch * maxd * 2);
+    for (int i = 0; i < 2; ++i) {
+        alloc((void **)&n->dY[i], (size_t)max_batch * maxd * 2);
+        alloc((void **)&n->dYT[i], (size_t)max_batch * maxd * 2);
+    }
     alloc((void **)&n->status, sizeof(int));
     if (e != cudaSuccess) {
         mlp_free(n);
@@ -845,7 +980,7 @@ ef_status ef_mlp_forward(ef_mlp_t n, const float *X, int ldx, float *Y, int ldy,
     if (ldx < n->nin || ldy < n->noutp || ldy % 2) return mlp_fail(EF_ERR_INVALID_ARG, "ldx >= nin, ldy >= padded nout (even)");
     if (B == 0) return EF_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    pack_input_kernel<<<grid_for(B * n->ninp), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, nullptr);
+    pack_input_kernel<false><<<dim3(n->ninp / TT, (unsigned)(B / TT)), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, nullptr);
     return mlp_forward_packed(n, B, Y, ldy, false, s);
 }
 
@@ -853,40 +988,49 @@ ef_status ef_mlp_forward(ef_mlp_t n, const float *X, int ldx, float *Y, int ldy,
 static ef_status mlp_grad_impl(ef_mlp_s *n, const float *X, int ldx, const float *T, int ldt, const float *wmask,
                                const float *roww, int64_t B, float *loss_dev, cudaStream_t s)
 {
-    pack_input_kernel<<<grid_for(B * n->ninp), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, n->XbT);
+    pack_input_kernel<true><<<dim3(n->ninp / TT, (unsigned)(B / TT)), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, n->XbT);
     // forward (last layer's fp32 output into dA as scratch)
     ef_status st = mlp_forward_packed(n, B, n->dA, n->noutp, true, s);
     if (st != EF_OK) return st;
-    // weighted count for the mean
-    float nw = (float)n->nout;
-    (void)nw;
     cudaError_t e = cudaMemsetAsync(loss_dev, 0, sizeof(float), s);
     if (e != cudaSuccess) return cuda_err(e, "loss reset");
-    mse_kernel<<<grid_for(B * n->noutp), 256, 0, s>>>(n->dA, n->noutp, T, ldt, wmask, roww, n->nout, n->noutp, B,
-                                                       1.f / ((float)B * (float)n->nout), n->dY, n->dYT, loss_dev);
+    mse_kernel<<<dim3(n->noutp / TT, (unsigned)(B / TT)), 256, 0, s>>>(n->dA, n->noutp, T, ldt, wmask, roww, n->nout, n->noutp, B,
+                                                                        1.f / ((float)B * (float)n->nout), n->dY[0], n->dYT[0],
+                                                                        loss_dev);
+    int cur = 0;
     // backward
     for (int l = n->nl - 1; l >= 0; --l) {
         const int out = n->dout[l], in = n->din[l];
         // dW_l = dPre_l^T A_{l-1}:  M = out, N = in, K = B; A = dPreT [out][B], B = A_{l-1}^T [in][B]
+        // (hi and lo halves: 2 in rows), folded to the gradient of the tied halves
         GemmArgs g{};
-        g.A = n->dYT;
+        g.A = n->dYT[cur];
         g.lda = (int)B;
         g.B = l == 0 ? n->XbT : n->actT[l - 1];
         g.ldb = (int)B;
         g.M = out;
         g.N = 2 * in;
         g.K = (int)B;
+        g.status = n->status;
         g.Cf = n->dW2;
         g.ldcf = 2 * in;
-        g.status = n->status;
-        e = gemm(g, s);
-        if (e != cudaSuccess) return cuda_err(e, "mlp grad gemm");
-        fold_split_kernel<<<grid_for((int64_t)out * in), 256, 0, s>>>(n->dW2, out, in, n->g + n->woff[l]);
-        rowsum_kernel<<<out, 256, 0, s>>>(n->dYT, B, out, n->g + n->boff[l]);
+        if (tc_tile(g)) {
+            e = gemm(g, s);
+            if (e != cudaSuccess) return cuda_err(e, "mlp grad gemm");
+            fold_split_kernel<<<grid_for((int64_t)out * in), 256, 0, s>>>(n->dW2, out, in, n->g + n->woff[l]);
+            rowsum_kernel<<<out, 256, 0, s>>>(n->dYT[cur], B, out, n->g + n->boff[l]);
+        } else {
+            g.Cf = n->g + n->woff[l];
+            g.ldcf = in;
+            g.db = n->g + n->boff[l];
+            e = gemm_sync<EPI_DW>(g, s);
+            if (e != cudaSuccess) return cuda_err(e, "mlp grad gemm");
+        }
         if (l == 0) break;
-        // dA_{l-1} = dPre_l W_l:  M = B, N = in, K = out; A = dPre [B][out], B = W^T [in][out]
+        // dPre_{l-1} = (dPre_l W_l) masked by pre_{l-1} > 0:  M = B, N = in, K = out; A = dPre [B][out],
+        // B = W^T [in][out].  The next layer's buffers: other CTAs still read this one's as operand.
         GemmArgs h{};
-        h.A = n->dY;
+        h.A = n->dY[cur];
         h.lda = out;
         h.B = n->WbT[l];
         h.ldb = out;
@@ -896,9 +1040,22 @@ static ef_status mlp_grad_impl(ef_mlp_s *n, const float *X, int ldx, const float
         h.Cf = n->dA;
         h.ldcf = in;
         h.status = n->status;
-        e = gemm(h, s);
-        if (e != cudaSuccess) return cuda_err(e, "mlp backprop gemm");
-        relu_back_kernel<<<grid_for(B * in), 256, 0, s>>>(n->dA, n->pre[l - 1], B, in, n->dY, n->dYT);
+        if (tc_tile(h)) {
+            e = gemm(h, s);
+            if (e != cudaSuccess) return cuda_err(e, "mlp backprop gemm");
+            relu_back_kernel<<<grid_for(B * in), 256, 0, s>>>(n->dA, n->pre[l - 1], B, in, n->dY[cur ^ 1], n->dYT[cur ^ 1]);
+        } else {
+            h.Cf = nullptr;
+            h.pre = n->pre[l - 1];
+            h.ldpre = in;
+            h.Cb = n->dY[cur ^ 1];
+            h.ldcb = in;
+            h.CbT = n->dYT[cur ^ 1];
+            h.ldcbt = (int)B;
+            e = gemm_sync<EPI_DA>(h, s);
+            if (e != cudaSuccess) return cuda_err(e, "mlp backprop gemm");
+        }
+        cur ^= 1;
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_err(e, "mlp backward");
