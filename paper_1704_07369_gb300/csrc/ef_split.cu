@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
             dg.template add_row<D, T>(s_m, s_mx, s_e2, s_eta, T(0), (D == 3 ? r / N : r) - N / 2, D == 3 ? r % N - N / 2 : 0, mn_f,
                                        T(3.0e38));
         }
+        cl.sync();                           // an Euler step in place: every row of F read before any is written
     }
     for (int i0 = (rank * kFinThreads + tid) * W; i0 < cell; i0 += C * kFinThreads * W) {
         T f[W], q[W], nu[W];

@@ -126,3 +126,31 @@ def test_split_calls_under_capture():
     for g, q in more:
         assert (q - ref[0]).abs().max().item() <= 2e-5 * ref[0].abs().max().item()
     plan.close()
+
+
+@pytest.mark.parametrize("N,n", [(16, 1), (24, 2), (40, 3), (48, 1), (48, 5)])
+def test_split_step_moments_are_of_the_old_state(N, n):
+    """The sums over F of a split FP32 step in place are over the state before the step: against FP64
+    sums of that state (a row in FP32, N terms of one sign: N u relative to the sum of magnitudes).
+    dt is large, so that a sum over a partly updated state shows."""
+    L, dt = 8.0, 0.3
+    host = np.stack(_cells(3, N, L, n))
+    F = torch.tensor(host, dtype=torch.float32, device="cuda")
+    old = F.double().cpu().numpy()
+    D = torch.zeros(n, ef.EF_DIAG_STRIDE, dtype=torch.float64, device="cuda")
+    plan = ef.Plan(3, N, L, ef.EF_KERNEL_HARD_SPHERE, 32, ef.EF_PREC_F32)
+    plan.euler(F, dt, diag=D, ncells=n)
+    torch.cuda.synchronize()
+    plan.close()
+    d, h = D.cpu().numpy(), 2 * L / N
+    v = (np.arange(N) - N // 2) * h
+    z, y, x = np.meshgrid(v, v, v, indexing="ij")
+    with np.errstate(divide="ignore", invalid="ignore"):
+        eta = np.where(old > 0, old * np.log(old), 0.0)
+    u = N * 2.0 ** -24
+    for k, w in ((0, old), (1, old * z), (2, old * y), (3, old * x), (4, 0.5 * old * (x * x + y * y + z * z))):
+        assert (np.abs(d[:, k] - h ** 3 * w.sum((1, 2, 3))) <= 2 * u * h ** 3 * np.abs(w).sum((1, 2, 3)) + 1e-12).all(), k
+    # the fast logarithm adds 2^-21.4 absolute (CUDA's bound for __logf in [0.5, 2]; relative 2 ulp elsewhere)
+    bound = (2 * u * np.abs(eta) + 2.0 ** -20 * np.abs(old)).sum((1, 2, 3))
+    assert (np.abs(d[:, 5] - h ** 3 * eta.sum((1, 2, 3))) <= h ** 3 * bound).all()
+    assert (d[:, 7] == old.min((1, 2, 3))).all()
