@@ -78,6 +78,8 @@ bool plan_view(const struct ef_plan_s *p, PlanView *out);
 ef_status ef_plan_create_batched_opt(int d, int64_t ncells, const int *N_host, double L, ef_kernel kernel, int R, ef_precision prec,
                               bool may_split, struct ef_plan_s **out);
 ef_status plan_create_padded(const ef_plan_desc *desc, struct ef_plan_s **out);
+// forward pass of n on the input that the last forward pass of `first` on this stream packed (ef_mlp.cu)
+ef_status mlp_forward_same_input(ef_mlp_t n, ef_mlp_t first, float *Y, int ldy, int64_t B, cudaStream_t s);
 
 // Axis-0 pencils per CTA of a C-CTA cluster (even, so that lane pairs never straddle CTAs) and the
 // bytes of one cluster's forward-spectrum workspace (N x NP complex).

@@ -18,6 +18,7 @@
 
 #include <mutex>
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -278,18 +279,28 @@ cudaError_t gemm_sync(const GemmArgs &g, cudaStream_t s)
 }
 
 // ------------------------------------------------------------ tcgen05 GEMM ---------------
-// The same product and epilogue on the 5th-generation tensor cores: one CTA of 4 warps per
-// 128 x TN tile of C, K in blocks of 64.  Thread 0 runs the pipeline: TMA loads (128-byte
-// swizzle) of the A and B tiles of a K block into one of TC_STAGES shared-memory stages, each
-// stage with a "full" mbarrier (TMA bytes arrived) and an "empty" one (its MMAs done, committed by
-// tcgen05.commit); tcgen05.mma kind::f16 (M = 128, N = TN, K = 16) accumulates in tensor memory;
-// a stage is refilled once the MMAs that read it are complete, after the next block's MMAs have
-// been queued.  The epilogue reads the accumulator with tcgen05.ld (warp w owns tensor-memory
-// lanes, i.e. rows, 32w .. 32w+31).  Every mbarrier wait is bounded.  A wait that gives up stops
-// the pipeline, records EF_ERR_TIMEOUT in the status word, waits (bounded) for the CTA's copies
-// and MMAs still in flight, and writes NaN for the tile without reading the accumulator; the
-// tensor memory is released in every case.
-constexpr int TC_BM = 128, TC_BK = 64, TC_STAGES = 4;
+// The same product and epilogue on the 5th-generation tensor cores, persistent: one CTA per SM works
+// through 128 x TN tiles of C (columns fastest, so that a row block of A is read from L2), K in blocks of
+// 64.  Six warps: a producer thread (TMA loads with 128-byte swizzle into a ring of shared-memory
+// stages), an MMA thread (tcgen05.mma kind::f16, M = 128, N = TN, K = 16), and four warps that write a
+// finished tile out while the next one is accumulated (two accumulators in tensor memory; warp w reads
+// lanes 32 (w % 4) ..).  A layer's product of 16384 cells is K = 1024 - 1920: 1 - 2 us of loads and MMAs a
+// tile against as long an epilogue, so the overlap is worth up to half.  Results leave through shared
+// memory, 64 or 128 contiguous bytes of a row at a time: written straight from the accumulator layout
+// (a thread per row) every store touched 32 half-used sectors.
+// Every mbarrier wait is bounded.  A wait that gives up stops its role (the others run out in turn),
+// records EF_ERR_TIMEOUT in the status word, the CTA's tiles from there on become NaN without a read of the
+// accumulator, copies and MMAs still in flight are waited for (bounded), and the tensor memory is
+// released in every case.
+constexpr int TC_BM = 128, TC_BK = 64, TC_THREADS = 192;
+constexpr int TC_SROW = 144;                     // staged row: 128 bytes, padded against bank conflicts
+template <int TN>
+__host__ __device__ constexpr int tc_stages() { return TN >= 256 ? 4 : TN >= 192 ? 5 : TN >= 128 ? 6 : 8; }
+template <int TN>
+__host__ __device__ constexpr size_t tc_smem()
+{
+    return (size_t)tc_stages<TN>() * (TC_BM + TN) * TC_BK * 2 + 4 * 32 * TC_SROW + 1024;
+}
 
 __device__ __forceinline__ uint64_t tc_sdesc(uint32_t addr)
 {
@@ -326,30 +337,37 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity)
 }
 
 template <int TN>
-__global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__ CUtensorMap tA,
-                                                         const __grid_constant__ CUtensorMap tB, const GemmArgs g)
+__global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_constant__ CUtensorMap tA,
+                                                                const __grid_constant__ CUtensorMap tB, const GemmArgs g)
 {
-    constexpr int A_BYTES = TC_BM * TC_BK * 2, B_BYTES = TN * TC_BK * 2, STAGE = A_BYTES + B_BYTES;
-    constexpr int TCOLS = TN <= 64 ? 64 : (TN <= 128 ? 128 : 256);     // tensor-memory columns
+    constexpr int A_BYTES = TC_BM * TC_BK * 2, B_BYTES = TN * TC_BK * 2, STAGE = A_BYTES + B_BYTES, ST = tc_stages<TN>();
+    constexpr int TCOLS = TN <= 64 ? 64 : (TN <= 128 ? 128 : 256);     // tensor-memory columns of one accumulator
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     unsigned char *tc_smem = (unsigned char *)(((uintptr_t)tc_raw + 1023) & ~(uintptr_t)1023);   // swizzle atoms
-    __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES];
+    __shared__ __align__(8) uint64_t full[ST], empty[ST], accf[2], acce[2], drain;
     __shared__ uint32_t tmem_base;
+    __shared__ int s_issued, s_used, s_fail;     // K blocks loaded, K blocks multiplied, a wait gave up
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TC_BM, n0 = blockIdx.x * TN;
-    const int nk = g.K / TC_BK;
+    const int nk = g.K / TC_BK, ncol = g.N / TN, ntiles = (g.M / TC_BM) * ncol;
     const uint32_t sbase = smem_u32(tc_smem);
 
-    if (warp == 0) {
+    if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
-                     "r"(TCOLS));
+                     "r"(2 * TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
     if (tid == 0) {
-        for (int i = 0; i < TC_STAGES; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[i])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[i])));
+        auto init = [](uint64_t *b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(b)), "r"(n)); };
+        for (int i = 0; i < ST; ++i) {
+            init(&full[i], 1);
+            init(&empty[i], 1);
         }
+        for (int i = 0; i < 2; ++i) {
+            init(&accf[i], 1);
+            init(&acce[i], 4);
+        }
+        init(&drain, 1);
+        s_issued = s_used = s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tA));
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tB));
@@ -359,128 +377,177 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
     const uint32_t tmem = tmem_base;
 
-    __shared__ int s_ok;
-    if (tid == 0) {
-        // pend[st]: a TMA load into stage st was issued and its "full" phase not yet waited for;
-        // ncommit[st]: commits of MMAs reading stage st.  Each stage has at most one outstanding
-        // phase of either barrier (a stage is refilled only after both were waited for), so every
-        // parity below names one phase.
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
+                const int m0 = t / ncol * TC_BM, n0 = t % ncol * TN;
+                for (int kb = 0; kb < nk; ++kb, ++it) {
+                    const int st = it % ST;
+                    if (it >= ST && !tc_wait(smem_u32(&empty[st]), (uint32_t)((it / ST - 1) & 1))) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t a0 = sbase + st * STAGE, b0 = a0 + A_BYTES, bar = smem_u32(&full[st]);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(STAGE));
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+                                 ::"r"(a0), "l"(&tA), "r"(kb * TC_BK), "r"(m0), "r"(bar) : "memory");
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+                                 ::"r"(b0), "l"(&tB), "r"(kb * TC_BK), "r"(n0), "r"(bar) : "memory");
+                }
+            }
+            s_issued = it;
+            if (!ok) atomicExch(&s_fail, 1);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int it = 0, j = 0;                   // K blocks so far, tiles so far
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++j) {
+                if (j >= 2 && !tc_wait(smem_u32(&acce[j & 1]), (uint32_t)((j / 2 - 1) & 1))) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+                const uint32_t acc_col = tmem + (uint32_t)(j & 1) * TCOLS;
+                for (int kb = 0; kb < nk; ++kb, ++it) {
+                    const int st = it % ST;
+                    if (!tc_wait(smem_u32(&full[st]), (uint32_t)((it / ST) & 1))) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+                    const uint32_t a0 = sbase + st * STAGE, b0 = a0 + A_BYTES;
+#pragma unroll
+                    for (int k16 = 0; k16 < TC_BK / 16; ++k16) {
+                        const uint64_t ad = tc_sdesc(a0 + k16 * 32), bd = tc_sdesc(b0 + k16 * 32);
+                        const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
+                        asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                                     ::"r"(acc_col), "l"(ad), "l"(bd), "r"(tc_idesc(TC_BM, TN)), "r"(acc));
+                    }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+                                 ::"r"(smem_u32(&empty[st])));
+                }
+                if (ok)
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+                                 ::"r"(smem_u32(&accf[j & 1])));
+            }
+            s_used = it;
+            if (!ok) {
+                // the MMAs queued so far, before their stages and accumulators go away
+                atomicExch(&s_fail, 1);
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(&drain)));
+                tc_wait(smem_u32(&drain), 0);
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
+        }
+    } else {
+        const int sub = warp & 3;                // tensor-memory lanes 32 sub ..
+        unsigned char *stg = tc_smem + ST * STAGE + sub * 32 * TC_SROW;
+        const float nan = __int_as_float(0x7fc00000);
         bool ok = true;
-        bool pend[TC_STAGES];
-        uint32_t fph[TC_STAGES], eph[TC_STAGES];
-        int ncommit[TC_STAGES];
-        int kb_last = -1;                                // the last K block whose MMAs were committed
-        auto issue = [&](int kb, int st) {
-            const uint32_t a0 = sbase + st * STAGE, b0 = a0 + A_BYTES, bar = smem_u32(&full[st]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(STAGE));
-            asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-                         ::"r"(a0), "l"(&tA), "r"(kb * TC_BK), "r"(m0), "r"(bar) : "memory");
-            asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-                         ::"r"(b0), "l"(&tB), "r"(kb * TC_BK), "r"(n0), "r"(bar) : "memory");
-            pend[st] = true;
-        };
-        for (int i = 0; i < TC_STAGES; ++i) {
-            fph[i] = eph[i] = 0;
-            pend[i] = false;
-            ncommit[i] = 0;
-            if (i < nk) issue(i, i);
-        }
-        for (int kb = 0; kb < nk; ++kb) {
-            const int st = kb % TC_STAGES;
-            if (!tc_wait(smem_u32(&full[st]), fph[st])) { ok = false; break; }
-            pend[st] = false;
-            fph[st] ^= 1;
+        int j = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
+            const int m0 = t / ncol * TC_BM + sub * 32, n0 = t % ncol * TN;
+            if (ok && !__all_sync(0xffffffffu, tc_wait(smem_u32(&accf[j & 1]), (uint32_t)((j / 2) & 1)))) {
+                ok = false;
+                if (lane == 0) atomicExch(&s_fail, 1);
+            }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-            const uint32_t a0 = sbase + st * STAGE, b0 = a0 + A_BYTES;
-#pragma unroll
-            for (int k16 = 0; k16 < TC_BK / 16; ++k16) {
-                const uint64_t ad = tc_sdesc(a0 + k16 * 32), bd = tc_sdesc(b0 + k16 * 32);
-                const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
-                asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             ::"r"(tmem), "l"(ad), "l"(bd), "r"(tc_idesc(TC_BM, TN)), "r"(acc));
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                         ::"r"(smem_u32(&empty[st])));
-            ++ncommit[st];
-            kb_last = kb;
-            const int nxt = kb - 1 + TC_STAGES;          // refill the stage of kb - 1
-            if (kb >= 1 && nxt < nk) {
-                const int pb = (kb - 1) % TC_STAGES;
-                if (!tc_wait(smem_u32(&empty[pb]), eph[pb])) { ok = false; break; }
-                eph[pb] ^= 1;
-                issue(nxt, pb);
-            }
-        }
-        // the last commit covers every MMA issued before it (tcgen05.commit tracks all prior
-        // asynchronous tcgen05 operations of this thread)
-        const int L = kb_last >= 0 ? kb_last % TC_STAGES : 0;
-        if (ok && kb_last >= 0) ok = tc_wait(smem_u32(&empty[L]), (uint32_t)((ncommit[L] - 1) & 1));
-        if (!ok) {
-            // a wait gave up: record it, then wait (again bounded) for this CTA's own copies and
-            // MMAs still in flight before the accumulator is released and the CTA exits
-            if (g.status) atomicCAS(g.status, 0, 5);     // EF_ERR_TIMEOUT
-            for (int i = 0; i < TC_STAGES; ++i)
-                if (pend[i]) tc_wait(smem_u32(&full[i]), fph[i]);
-            if (kb_last >= 0) tc_wait(smem_u32(&empty[L]), (uint32_t)((ncommit[L] - 1) & 1));
-        }
-        s_ok = ok ? 1 : 0;
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-    }
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-    const bool ok = s_ok != 0;
-
-    const int row = m0 + warp * 32 + lane;
-    const float bad = __int_as_float(0x7fc00000);
+            const uint32_t acc = tmem + (uint32_t)(j & 1) * TCOLS + ((uint32_t)(sub * 32) << 16);
 #pragma unroll 1
-    for (int c0 = 0; c0 < TN; c0 += 8) {
-        uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (ok) {            // CTA-uniform: after a give-up the accumulator is not read
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + c0;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                         : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-        }
-        const int col = n0 + c0;
-        float v[8];
+            for (int c0 = 0; c0 < TN; c0 += 32) {
+                uint32_t r[32];
+                if (ok) {                        // warp-uniform: after a give-up the accumulator is not read
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+                                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                                 : "r"(acc + c0));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
+                    if (c0 + 32 == TN) {         // the accumulator is read: the MMA thread may start on it again
+                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
+                        __syncwarp();
+                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acce[j & 1])) : "memory");
+                    }
+                } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            v[j] = ok ? __uint_as_float(r[j]) : bad;
-            if (g.bias) v[j] += g.bias[col + j];
-        }
-        if (g.Cf) {
-            float4 *d = reinterpret_cast<float4 *>(g.Cf + (size_t)row * g.ldcf + col);
-            d[0] = make_float4(v[0], v[1], v[2], v[3]);
-            d[1] = make_float4(v[4], v[5], v[6], v[7]);
-        }
-        if (g.relu) {
+                    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(nan);
+                }
+                const int col = n0 + c0;
+                float v[32];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = fmaxf(v[j], 0.f);
-        }
-        bf16 hi[8], lo[8];
+                for (int i = 0; i < 32; i += 4) {
+                    const float4 b = g.bias ? __ldg(reinterpret_cast<const float4 *>(g.bias + col + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[i] = __uint_as_float(r[i]) + b.x;
+                    v[i + 1] = __uint_as_float(r[i + 1]) + b.y;
+                    v[i + 2] = __uint_as_float(r[i + 2]) + b.z;
+                    v[i + 3] = __uint_as_float(r[i + 3]) + b.w;
+                }
+                if (g.Cf) {
+                    __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            hi[j] = __float2bfloat16(v[j]);
-            lo[j] = __float2bfloat16(v[j] - __bfloat162float(hi[j]));
-        }
-        if (g.Cb) {
-            *reinterpret_cast<uint4 *>(g.Cb + (size_t)row * g.ldcb + col) = *reinterpret_cast<const uint4 *>(hi);
-            if (g.lo_off)
-                *reinterpret_cast<uint4 *>(g.Cb + (size_t)row * g.ldcb + g.lo_off + col) = *reinterpret_cast<const uint4 *>(lo);
-        }
-        if (g.CbT) {
+                    for (int i = 0; i < 8; ++i)
+                        *reinterpret_cast<float4 *>(stg + lane * TC_SROW + i * 16) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    __syncwarp();
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                g.CbT[(size_t)(col + j) * g.ldcbt + row] = hi[j];
-                if (g.lo_off) g.CbT[(size_t)(g.lo_off + col + j) * g.ldcbt + row] = lo[j];
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = i * 4 + (lane >> 3), pc = lane & 7;
+                        *reinterpret_cast<float4 *>(g.Cf + (size_t)(m0 + rr) * g.ldcf + col + pc * 4) =
+                            *reinterpret_cast<const float4 *>(stg + rr * TC_SROW + pc * 16);
+                    }
+                }
+                if (!g.Cb && !g.CbT) continue;
+                if (g.relu) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f);
+                }
+                bf16 hi[32], lo[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    hi[i] = __float2bfloat16(v[i]);
+                    lo[i] = __float2bfloat16(v[i] - __bfloat162float(hi[i]));
+                }
+                if (g.Cb) {
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        *reinterpret_cast<uint4 *>(stg + lane * TC_SROW + i * 16) = *reinterpret_cast<const uint4 *>(hi + 8 * i);
+                        *reinterpret_cast<uint4 *>(stg + lane * TC_SROW + 64 + i * 16) = *reinterpret_cast<const uint4 *>(lo + 8 * i);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {            // 64 bytes of the hi half and 64 of the lo half of a row
+                        const int rr = i * 4 + (lane >> 3), pc = lane & 7, half = pc >> 2;
+                        if (half == 0 || g.lo_off)
+                            *reinterpret_cast<uint4 *>(g.Cb + (size_t)(m0 + rr) * g.ldcb + half * g.lo_off + col + (pc & 3) * 8) =
+                                *reinterpret_cast<const uint4 *>(stg + rr * TC_SROW + pc * 16);
+                    }
+                }
+                if (g.CbT) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        g.CbT[(size_t)(col + i) * g.ldcbt + m0 + lane] = hi[i];
+                        if (g.lo_off) g.CbT[(size_t)(g.lo_off + col + i) * g.ldcbt + m0 + lane] = lo[i];
+                    }
+                }
             }
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TCOLS));
+    if (s_fail) {
+        if (tid == 0) {
+            if (g.status) atomicCAS(g.status, 0, 5);     // EF_ERR_TIMEOUT
+            for (int it = s_used; it < s_issued; ++it) tc_wait(smem_u32(&full[it % ST]), (uint32_t)((it / ST) & 1));
+        }
+        __syncthreads();
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * TCOLS));
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against the driver)
@@ -512,10 +579,24 @@ bool tile_map(CUtensorMap *m, const bf16 *base, int rows, int K, int ld, int box
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int device_sms()
+{
+    static std::atomic<int> sms{0};
+    int n = sms.load(std::memory_order_relaxed);
+    if (n == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (n <= 0) n = 1;
+        sms.store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
 template <int TN>
 cudaError_t gemm_tc(const GemmArgs &g, bool *used, cudaStream_t s)
 {
-    constexpr size_t smem = (size_t)TC_STAGES * (TC_BM * TC_BK * 2 + TN * TC_BK * 2) + 1024;
+    constexpr size_t smem = tc_smem<TN>();
     *used = false;
     CUtensorMap tA, tB;
     if (!tile_map(&tA, g.A, g.M, g.K, g.lda, TC_BM) || !tile_map(&tB, g.B, g.N, g.K, g.ldb, TN)) return cudaSuccess;
@@ -529,30 +610,34 @@ cudaError_t gemm_tc(const GemmArgs &g, bool *used, cudaStream_t s)
         if (e != cudaSuccess) return e;
         __atomic_fetch_or(&set_on, bit, __ATOMIC_ACQ_REL);
     }
-    dim3 grid(g.N / TN, g.M / TC_BM);
-    gemm_tc_kernel<TN><<<grid, 128, smem, s>>>(tA, tB, g);
+    const int64_t tiles = (int64_t)(g.M / TC_BM) * (g.N / TN);
+    gemm_tc_kernel<TN><<<(int)std::min<int64_t>(tiles, device_sms()), TC_THREADS, smem, s>>>(tA, tB, g);
     *used = true;
     return cudaGetLastError();
 }
 
-// the tcgen05 kernel's widest N tile that still gives every SM a tile, 0 where the product is not its
-// (small products keep the 64 x 64 mma.sync kernel, whose many CTAs fill the device)
+// The tcgen05 kernel's tile width, 0 where the product is not its (small products keep the 64 x 64
+// mma.sync kernel, whose many CTAs fill the device).  The width with the shortest run of the busiest
+// SM: rounds of tiles, each as long as its columns and about 32 more (a narrow tile reads its rows of A
+// from shared memory for fewer columns).
 int tc_tile(const GemmArgs &g)
 {
     const bool aligned = g.lda % 8 == 0 && g.ldb % 8 == 0 && (!g.Cf || g.ldcf % 4 == 0) && (!g.Cb || g.ldcb % 8 == 0) &&
-                         g.lo_off % 8 == 0;
+                         g.lo_off % 8 == 0 && ((uintptr_t)g.bias | (uintptr_t)g.Cf | (uintptr_t)g.Cb) % 16 == 0;
     if (g.M % TC_BM || g.K % TC_BK || !aligned) return 0;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
+    const int64_t sms = device_sms(), mt = g.M / TC_BM;
+    if (g.N % 64 || mt * (g.N / 64) < sms) return 0;
+    int best = 0;
+    int64_t cost = 0;
+    for (int tn : {256, 192, 128, 64}) {
+        if (g.N % tn) continue;
+        const int64_t c = (mt * (g.N / tn) + sms - 1) / sms * (tn + 32);
+        if (!best || c < cost) {
+            best = tn;
+            cost = c;
+        }
     }
-    const int64_t mt = g.M / TC_BM;
-    for (int tn : {256, 192, 128, 64})
-        if (g.N % tn == 0 && mt * (g.N / tn) >= sms) return tn;
-    return 0;
+    return best;
 }
 
 // tcgen05 for the shapes it tiles (M multiple of 128, K of 64, N of 64, 16-byte aligned rows) with at
@@ -590,8 +675,8 @@ template <bool TR>
 __global__ void __launch_bounds__(256) pack_input_kernel(const float *X, int ldx, int nin, int ninp, int64_t B, bf16 *Xb, bf16 *XbT)
 {
     __shared__ bf16 th[TR ? TT : 1][TTL], tl[TR ? TT : 1][TTL];
-    const int64_t b0 = (int64_t)blockIdx.y * TT;
-    const int j0 = blockIdx.x * TT;
+    const int64_t b0 = (int64_t)blockIdx.x * TT;
+    const int j0 = blockIdx.y * TT;
     for (int i = threadIdx.x; i < TT * TT / 2; i += blockDim.x) {
         const int r = i / (TT / 2), c = (i % (TT / 2)) * 2, j = j0 + c;
         const int64_t b = b0 + r;
@@ -631,8 +716,8 @@ __global__ void __launch_bounds__(256) mse_kernel(const float *Y, int ldy_pred, 
                            int nout, int noutp, int64_t B, float inv_count, bf16 *dY, bf16 *dYT, float *loss)
 {
     __shared__ bf16 th[TT][TTL];
-    const int64_t b0 = (int64_t)blockIdx.y * TT;
-    const int j0 = blockIdx.x * TT;
+    const int64_t b0 = (int64_t)blockIdx.x * TT;
+    const int j0 = blockIdx.y * TT;
     float acc = 0.f;
     for (int i = threadIdx.x; i < TT * TT / 2; i += blockDim.x) {
         const int r = i / (TT / 2), c = (i % (TT / 2)) * 2;
@@ -800,12 +885,12 @@ void mlp_free(ef_mlp_s *n)
     delete n;
 }
 
-// forward pass for batch B (multiple of 64) from the packed input n->Xb
-ef_status mlp_forward_packed(ef_mlp_s *n, int64_t B, float *Yout, int ldy, bool keep_T, cudaStream_t s)
+// forward pass for batch B (multiple of 64) from the packed input Xb
+ef_status mlp_forward_packed(ef_mlp_s *n, const bf16 *Xb, int64_t B, float *Yout, int ldy, bool keep_T, cudaStream_t s)
 {
     for (int l = 0; l < n->nl; ++l) {
         GemmArgs g{};
-        g.A = l == 0 ? n->Xb : n->act[l - 1];
+        g.A = l == 0 ? Xb : n->act[l - 1];
         g.lda = 2 * n->din[l];
         g.B = n->Wb[l];
         g.ldb = 2 * n->din[l];
@@ -830,6 +915,16 @@ ef_status mlp_forward_packed(ef_mlp_s *n, int64_t B, float *Yout, int ldy, bool 
 }
 
 }  // namespace
+
+namespace ef {
+
+ef_status mlp_forward_same_input(ef_mlp_t n, ef_mlp_t first, float *Y, int ldy, int64_t B, cudaStream_t s)
+{
+    if (n->ninp != first->ninp || B > n->max_batch || B > first->max_batch) return mlp_fail(EF_ERR_INVALID_ARG, "networks of one input");
+    return mlp_forward_packed(n, first->Xb, B, Y, ldy, false, s);
+}
+
+}  // namespace ef
 
 extern "C" {
 
@@ -980,21 +1075,21 @@ ef_status ef_mlp_forward(ef_mlp_t n, const float *X, int ldx, float *Y, int ldy,
     if (ldx < n->nin || ldy < n->noutp || ldy % 2) return mlp_fail(EF_ERR_INVALID_ARG, "ldx >= nin, ldy >= padded nout (even)");
     if (B == 0) return EF_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    pack_input_kernel<false><<<dim3(n->ninp / TT, (unsigned)(B / TT)), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, nullptr);
-    return mlp_forward_packed(n, B, Y, ldy, false, s);
+    pack_input_kernel<false><<<dim3((unsigned)(B / TT), n->ninp / TT), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, nullptr);
+    return mlp_forward_packed(n, n->Xb, B, Y, ldy, false, s);
 }
 
 // loss and gradients (into the MLP's gradient buffer); optionally the Adam update
 static ef_status mlp_grad_impl(ef_mlp_s *n, const float *X, int ldx, const float *T, int ldt, const float *wmask,
                                const float *roww, int64_t B, float *loss_dev, cudaStream_t s)
 {
-    pack_input_kernel<true><<<dim3(n->ninp / TT, (unsigned)(B / TT)), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, n->XbT);
+    pack_input_kernel<true><<<dim3((unsigned)(B / TT), n->ninp / TT), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, n->XbT);
     // forward (last layer's fp32 output into dA as scratch)
-    ef_status st = mlp_forward_packed(n, B, n->dA, n->noutp, true, s);
+    ef_status st = mlp_forward_packed(n, n->Xb, B, n->dA, n->noutp, true, s);
     if (st != EF_OK) return st;
     cudaError_t e = cudaMemsetAsync(loss_dev, 0, sizeof(float), s);
     if (e != cudaSuccess) return cuda_err(e, "loss reset");
-    mse_kernel<<<dim3(n->noutp / TT, (unsigned)(B / TT)), 256, 0, s>>>(n->dA, n->noutp, T, ldt, wmask, roww, n->nout, n->noutp, B,
+    mse_kernel<<<dim3((unsigned)(B / TT), n->noutp / TT), 256, 0, s>>>(n->dA, n->noutp, T, ldt, wmask, roww, n->nout, n->noutp, B,
                                                                         1.f / ((float)B * (float)n->nout), n->dY[0], n->dYT[0],
                                                                         loss_dev);
     int cur = 0;
