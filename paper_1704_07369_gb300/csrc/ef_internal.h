@@ -62,6 +62,9 @@ struct CollideArgs {
     int nsplit = 1;           // parts per cell (>= 1): a work item is one part, with its share of the ops
     void *part = nullptr;     // nsplit > 1: [cell][nsplit + 1][N^d] gain of each part, then nu; summed and
                               // written out by the finishing kernel (ef_split.cu)
+    int fin_ctas = 1;         // its CTAs per cell, and their meeting place: arrivals [cell], zero between
+    void *fin = nullptr;      // launches; fin_off bytes on, the CTAs' diagnostics [cell][fin_ctas][kDiag]
+    size_t fin_off = 0;
 };
 
 // Arguments of the low-mode feature kernel (one launch per size class).

@@ -47,6 +47,7 @@ cudaError_t rg_split_setup_f32(int N, int v, size_t smem, int cluster, int tpb, 
 cudaError_t rg_split_launch_f32(int N, int v, const CollideArgs &a, int grid_clusters, int tpb, size_t smem, cudaStream_t s);
 // Q / F + dt Q and diagnostics from the parts of a split collide launch (ef_split.cu)
 cudaError_t split_finish_setup(int prec, int d);
+int split_finish_ctas(int prec, int d, int N, int64_t n, int sms);
 cudaError_t split_finish_launch(int prec, int d, int N, const CollideArgs &a, cudaStream_t s);
 
 EF_DECLARE_VARIANT(f32_2d)

@@ -261,6 +261,8 @@ struct ClassPlan {
     int pick_s = 1;
     void *d_part = nullptr;             // gains of the parts of split launches, kPartSlots workspaces
     size_t part_bytes = 0;              // of one workspace
+    void *d_fin = nullptr;              // arrivals and diagnostics of the finishing launches, kPartSlots of them
+    size_t fin_off = 0, fin_bytes = 0;  // diagnostics behind the arrivals, bytes of one
     size_t smem = 0;
     int max_clusters = 0;
     int ndir = 0, nops = 0;              // op count of the active mode
@@ -628,13 +630,17 @@ void cache_store(const std::string &key, int C, int tpb, int sg, int pf, int pr,
     std::fclose(f);
 }
 
+// arrivals of n cells, and the diagnostics of the CTAs of at most n (split_finish_ctas)
+size_t fin_offset(int64_t n) { return ((size_t)n * sizeof(int) + 255) / 256 * 256; }
+size_t fin_diag_bytes(int64_t n, int sms) { return ((size_t)std::max<int64_t>(n, 4 * (int64_t)sms) * ef::kDiag * 8 + 255) / 256 * 256; }
+
 // Plan-time autotuner: time every candidate shape (and the L1 prefetch on / off), as an Euler step
 // with the diagnostics, on a scratch batch of up to 512 cells, then the three fastest again on a batch of ncells_tune cells (the size
 // class's own count, up to 2048: the tail of the last round of clusters and the packing of clusters
 // on the SMs depend on it), and keep the fastest of those.  Results are cached per device and
 // discretisation in the file named by EF_AUTOTUNE_CACHE when it is set; EF_AUTOTUNE=0 skips the
 // timing and takes the smallest cluster.
-ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool may_split)
+ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool may_split, int sms)
 {
     std::string why;
     std::vector<Shape> shapes = candidate_shapes(ds, cp.N, why);
@@ -686,7 +692,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
     const int d = ds.d;
     const int64_t cell = d == 3 ? (int64_t)cp.N * cp.N * cp.N : (int64_t)cp.N * cp.N;
     const size_t el = ds.prec == EF_PREC_F32 ? 4 : 8;
-    void *F = nullptr, *Q = nullptr, *sgws = nullptr, *fhws = nullptr, *parts_ws = nullptr;
+    void *F = nullptr, *Q = nullptr, *sgws = nullptr, *fhws = nullptr, *parts_ws = nullptr, *fin_ws = nullptr;
     double *dgws = nullptr;
     cudaStream_t st = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -711,6 +717,10 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
             if (S > 1) part_cells = std::max<int64_t>(part_cells, ncells_tune * (S + 1));
         }
     if (e == cudaSuccess && part_cells) e = cudaMalloc(&parts_ws, (size_t)part_cells * cell * el);
+    const size_t fin_bytes = fin_offset(ncells_tune) + fin_diag_bytes(ncells_tune, sms);
+    if (e == cudaSuccess && part_cells) e = cudaMalloc(&fin_ws, fin_bytes);
+    if (e == cudaSuccess && part_cells) e = cudaMemset(fin_ws, 0, fin_bytes);
+    if (e == cudaSuccess && part_cells) e = cudaDeviceSynchronize();
     double best = 1e30;
     Shape best_sh = shapes[0];
     int best_pf = 0, best_split = 1;
@@ -746,6 +756,9 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
         a.prefetch = pfv;
         a.nsplit = split;
         a.part = parts_ws;
+        a.fin = fin_ws;
+        a.fin_off = fin_offset(ncells_tune);
+        if (split > 1) a.fin_ctas = ef::split_finish_ctas(ds.prec == EF_PREC_F32 ? 0 : 1, d, cp.N, nc, sms);
         tmin = 1e30;
         cudaError_t r = cudaSuccess;
         for (int rep = 0; rep < 4 && r == cudaSuccess; ++rep) {
@@ -819,6 +832,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
     cudaFree(fhws);
     cudaFree(dgws);
     cudaFree(parts_ws);
+    cudaFree(fin_ws);
     if (st) cudaStreamDestroy(st);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -843,7 +857,7 @@ void *upload_table(const std::vector<double> &h, cudaError_t &err)
     return p;
 }
 
-ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split)
+ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split, int sms)
 {
     const int N = cp.N, d = ds.d;
     const int H = N / 2 + 1, N1 = d == 3 ? N : 1, NP = N1 * H;
@@ -959,7 +973,7 @@ ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split)
         if (e != cudaSuccess) return cuda_fail(e, "feature table");
         cp.nfeat = (int)modes.size() / 3;
     }
-    return choose_shape(ds, cp, cp.ncells > 0 ? std::min<int64_t>(cp.ncells, 2048) : 0, may_split);
+    return choose_shape(ds, cp, cp.ncells > 0 ? std::min<int64_t>(cp.ncells, 2048) : 0, may_split, sms);
 }
 
 // Workspaces of one class for every cluster that can be resident at once (max_clusters, fixed by
@@ -972,14 +986,18 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
     const int64_t cell = (int64_t)cp.N * cp.N * (ds.d == 3 ? cp.N : 1);
     std::vector<Shape> used(1, cp.cur);
     if (!p->batched) used.insert(used.end(), cp.shapes.begin(), cp.shapes.end());
-    int64_t clusters = 1, sg_clusters = 0, part_cells = 0;
+    int64_t clusters = 1, sg_clusters = 0, part_cells = 0, fin_cells = 0;      // fin_cells: of a split launch
     for (const Shape &sh : used) {
         clusters = std::max<int64_t>(clusters, sh.max_clusters);
         if (sh.sg_global) sg_clusters = std::max<int64_t>(sg_clusters, sh.max_clusters);
         // uniform: n cells in S parts, n S at most the resident clusters, and nu: n (S + 1) <= 3/2 of them
+        if (!p->batched && max_split(ds, cp, sh, 1) > 1) fin_cells = std::max<int64_t>(fin_cells, sh.max_clusters);
         if (!p->batched && max_split(ds, cp, sh, 1) > 1) part_cells = std::max<int64_t>(part_cells, sh.max_clusters + (sh.max_clusters + 1) / 2);
     }
-    if (p->batched && cp.split > 1) part_cells = cp.ncells * (cp.split + 1);
+    if (p->batched && cp.split > 1) {
+        part_cells = cp.ncells * (cp.split + 1);
+        fin_cells = cp.ncells;
+    }
     cudaError_t e = cudaMalloc(&cp.d_fh, (size_t)clusters * ef::collide_fh_bytes(ds.prec, ds.d, cp.N));
     if (e != cudaSuccess) { cp.d_fh = nullptr; return cuda_fail(e, "spectrum workspace"); }
     cp.fh_slots = clusters;
@@ -993,6 +1011,13 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
         cp.part_bytes = (cp.part_bytes + 255) / 256 * 256;
         e = cudaMalloc(&cp.d_part, kPartSlots * cp.part_bytes);
         if (e != cudaSuccess) { cp.d_part = nullptr; return cuda_fail(e, "part workspace"); }
+        cp.fin_off = fin_offset(fin_cells);
+        cp.fin_bytes = cp.fin_off + fin_diag_bytes(fin_cells, p->sms);
+        e = cudaMalloc(&cp.d_fin, kPartSlots * cp.fin_bytes);
+        if (e != cudaSuccess) { cp.d_fin = nullptr; return cuda_fail(e, "part workspace"); }
+        e = cudaMemset(cp.d_fin, 0, kPartSlots * cp.fin_bytes);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();      // whatever stream the first call is on
+        if (e != cudaSuccess) return cuda_fail(e, "part workspace");
     }
     return EF_OK;
 }
@@ -1021,6 +1046,7 @@ void destroy_plan(ef_plan_s *p)
         cudaFree(cp.d_sg);
         cudaFree(cp.d_fh);
         cudaFree(cp.d_part);
+        cudaFree(cp.d_fin);
     }
     if (p->split_done) cudaEventDestroy(p->split_done);
     cudaFree(p->d_all_off);
@@ -1230,6 +1256,11 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         a.sg_ws = cp.d_sg;
         a.nsplit = S;
         a.part = static_cast<unsigned char *>(cp.d_part) + (slot > 0 ? slot : 0) * cp.part_bytes;
+        if (S > 1) {
+            a.fin = static_cast<unsigned char *>(cp.d_fin) + (slot > 0 ? slot : 0) * cp.fin_bytes;
+            a.fin_off = cp.fin_off;
+            a.fin_ctas = ef::split_finish_ctas(ds.prec == EF_PREC_F32 ? 0 : 1, ds.d, cp.N, n, p->sms);
+        }
         a.fh_ws = cp.d_fh;
         a.npc = ef::collide_npc_v(ds.prec, ds.d, cp.N, sh.cluster, sh.occ);
         a.out_mode = mode;
@@ -1263,7 +1294,7 @@ ef_status finish_plan(ef_plan_s *p)
     e = cudaMemset(p->d_status, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "status word");
     for (ClassPlan &cp : p->classes) {
-        ef_status st = build_class(p->desc, cp, p->may_split);
+        ef_status st = build_class(p->desc, cp, p->may_split, p->sms);
         if (st != EF_OK) return st;
         st = alloc_workspaces(p, cp);
         if (st != EF_OK) return st;

@@ -6,13 +6,20 @@
 // through all of its cell's ops; split, the ops of one cell run on several clusters at once, each
 // repeating the forward transform, and their partial gains meet here.  The parts are read back from
 // L2 (a part is N^d values, all parts of a launch at most the clusters' worth of cells), eight loads
-// in flight a thread, in part order, so the result does not depend on timing.  One cluster of CTAs per
-// cell: the diagnostics meet in distributed shared memory.
+// in flight a thread, in part order, so the result does not depend on timing.  A cell's rows are spread
+// over as many CTAs as fill the device (split_finish_ctas): an FP64 warp instruction takes a
+// sub-partition 64 cycles, and a point's logarithm and sums are about 65 of them.  A CTA owns whole
+// rows, so that a step in place may write them behind its own reads alone; the diagnostics of the
+// CTAs meet in global memory, summed in CTA order by whichever CTA arrives last.
+// One cluster of at most eight CTAs per cell, the diagnostics in distributed shared memory, took 88 us
+// for an FP64 cell of N = 32, 13 us for an FP64 2D cell of N = 16 and 17 us for the 49 parts of an FP32
+// cell of N = 32.
 //
-// Measured, unsplit against split with the shape that pick_shape chooses (ef_plan.cpp): Q of one FP32
-// cell of N = 32 (Maxwell, 49 ops) 427 -> 31 us; 100 Euler steps with diagnostics of one FP64 2D cell of
-// N = 16 16.8 -> 4.7 ms; two such steps of one FP64 cell of N = 32 14.0 -> 1.11 ms; two SSP-RK3 steps of
-// four FP64 2D cells of N = 64 5.3 -> 1.17 ms.
+// Measured, unsplit one-line-per-thread kernels against split with the shape that pick_shape chooses
+// (ef_plan.cpp) and the present kernels: Q of one FP32 cell of N = 32 (Maxwell, 49 ops) 427 -> 25 us; 100
+// Euler steps with diagnostics of one FP64 2D cell of N = 16 16.8 -> 2.46 ms; two such steps of one FP64
+// cell of N = 32 14.0 -> 0.79 ms; two SSP-RK3 steps of four FP64 2D cells of N = 64 5.3 -> 0.80 ms.
+#include <algorithm>
 #include <type_traits>
 
 #include "ef_collide_impl.cuh"
@@ -21,32 +28,54 @@
 namespace ef {
 namespace {
 
-constexpr int kFinThreads = 256;
+constexpr int kFinThreads = 128;     // one warp per sub-partition
 
-template <typename T>
-struct FinVec;
-template <>
-struct FinVec<float> {
+// values per thread and pass (split_finish_ctas has them too): 2D FP64 cells are small, so one
+template <typename T, int D>
+struct FinVec {
     using type = float4;
     static constexpr int W = 4;
 };
 template <>
-struct FinVec<double> {
+struct FinVec<double, 3> {
     using type = double2;
     static constexpr int W = 2;
 };
+template <>
+struct FinVec<double, 2> {
+    using type = double;
+    static constexpr int W = 1;
+};
+
+// v[k] of all lanes summed, k < 8, with 9 additions a lane in place of 40: lanes 4 k .. 4 k + 3 return sum k
+__device__ __forceinline__ double warp_sum8(double (&v)[8], int lane)
+{
+#pragma unroll
+    for (int h = 4, sh = 16; h >= 1; h >>= 1, sh >>= 1) {
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const bool up = lane & sh;
+            const double keep = up ? v[j + h] : v[j], send = up ? v[j] : v[j + h];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a, int N)
 {
-    using V = typename FinVec<T>::type;
-    constexpr int W = FinVec<T>::W;
+    using V = typename FinVec<T, D>::type;
+    constexpr int W = FinVec<T, D>::W;
     constexpr bool FFD = sizeof(T) == 4 && D == 3;
     constexpr bool ROWS = sizeof(T) == 4;    // sums over F row by row
     using DG = std::conditional_t<FFD, DiagF, Diag>;
-    cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int C = a.fin_ctas, rank = (int)(blockIdx.x % C);
     const int64_t c = blockIdx.x / C;
+    const int nrow = D == 3 ? N * N : N, rpc = (nrow + C - 1) / C;
+    const int r0 = min(rank * rpc, nrow), r1 = min(r0 + rpc, nrow);     // rows of this CTA
     const int S = a.nsplit;
     const int cell = (D == 3 ? N * N : N) * N;
     const int64_t coff = a.cell_off ? a.cell_off[c] : c * (int64_t)cell;
@@ -63,7 +92,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
     if (ROWS && a.diag) {
         // FP32: the sums over F by rows, in the order of emit_row, so that a cell's moments do not
         // depend on whether its launch was split
-        for (int r = rank * kFinThreads + tid; r < (D == 3 ? N * N : N); r += C * kFinThreads) {
+        for (int r = r0 + tid; r < r1; r += kFinThreads) {
             T s_m = 0, s_mx = 0, s_e2 = 0, s_eta = 0, mn_f = F[r * N];
 #pragma unroll 4
             for (int n0 = 0; n0 < N; n0 += W) {
@@ -82,9 +111,9 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
             dg.template add_row<D, T>(s_m, s_mx, s_e2, s_eta, T(0), (D == 3 ? r / N : r) - N / 2, D == 3 ? r % N - N / 2 : 0, mn_f,
                                        T(3.0e38));
         }
-        cl.sync();                           // an Euler step in place: every row of F read before any is written
+        __syncthreads();                     // an Euler step in place: the CTA's rows of F read before any is written
     }
-    for (int i0 = (rank * kFinThreads + tid) * W; i0 < cell; i0 += C * kFinThreads * W) {
+    for (int i0 = r0 * N + tid * W; i0 < r1 * N; i0 += kFinThreads * W) {
         T f[W], q[W], nu[W];
         *reinterpret_cast<V *>(f) = *reinterpret_cast<const V *>(F + i0);
         *reinterpret_cast<V *>(nu) = __ldcg(reinterpret_cast<const V *>(part + (int64_t)S * cell + i0));
@@ -151,75 +180,103 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
     if (!a.diag) return;
 
     auto merge = [](int k, double v, double u) { return (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u); };
+    auto extreme = [](int k, auto x) {
 #pragma unroll
-    for (int k = 0; k < kDiag; ++k) {
-        double v;
-        if constexpr (FFD) {
-            if (k < 7) {
-                FF x = dg.sum[k];
-#pragma unroll
-                for (int sh = 16; sh > 0; sh >>= 1)
-                    x = ff_merge(x, FF{__shfl_xor_sync(0xffffffffu, x.hi, sh), __shfl_xor_sync(0xffffffffu, x.lo, sh)});
-                v = ff_value(x);
-            } else {
-                float x = k == 7 ? dg.min_f : k == 8 ? dg.max_nu : dg.min_out;
-#pragma unroll
-                for (int sh = 16; sh > 0; sh >>= 1) {
-                    const float u = __shfl_xor_sync(0xffffffffu, x, sh);
-                    x = k == 8 ? fmaxf(x, u) : fminf(x, u);
-                }
-                v = x;
-            }
-        } else {
-            v = k < 7 ? dg.sum[k] : k == 7 ? dg.min_f : k == 8 ? dg.max_nu : dg.min_out;
-#pragma unroll
-            for (int sh = 16; sh > 0; sh >>= 1) v = merge(k, v, __shfl_xor_sync(0xffffffffu, v, sh));
+        for (int sh = 16; sh > 0; sh >>= 1) {
+            const auto u = __shfl_xor_sync(0xffffffffu, x, sh);
+            x = k == 8 ? fmax(x, u) : fmin(x, u);
         }
-        if (lane == 0) red[warp][k] = v;
+        return x;
+    };
+    if constexpr (FFD) {
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            FF x = dg.sum[k];
+#pragma unroll
+            for (int sh = 16; sh > 0; sh >>= 1)
+                x = ff_merge(x, FF{__shfl_xor_sync(0xffffffffu, x.hi, sh), __shfl_xor_sync(0xffffffffu, x.lo, sh)});
+            if (lane == 0) red[warp][k] = ff_value(x);
+        }
+    } else {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) v[k] = dg.sum[k];
+        v[7] = 0.0;
+        const double t = warp_sum8(v, lane);
+        if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
+    }
+    {
+        const double mf = extreme(7, dg.min_f), mx = extreme(8, dg.max_nu), mo = extreme(9, dg.min_out);
+        if (lane == 0) {
+            red[warp][7] = mf;
+            red[warp][8] = mx;
+            red[warp][9] = mo;
+        }
     }
     __syncthreads();
-    if (tid < kDiag) {
-        double v = red[0][tid];
-        for (int w = 1; w < kFinThreads / 32; ++w) v = merge(tid, v, red[w][tid]);
-        red[kFinThreads / 32][tid] = v;
-    }
-    cl.sync();
-    if (rank == 0 && tid < kDiag) {
-        const int k = tid;
-        double v = red[kFinThreads / 32][k];
-        for (int r = 1; r < C; ++r) v = merge(k, v, cl.map_shared_rank(&red[0][0], r)[(kFinThreads / 32) * kDiag + k]);
+    auto finish = [&](int k, double v) {
         const double hd = (D == 3) ? a.h * a.h * a.h : a.h * a.h;
         if (k == 0 || k == 5) v *= hd;
         else if (k >= 1 && k <= 3) v *= hd * a.h;
         else if (k == 4) v *= 0.5 * hd * a.h * a.h;
         if (D == 2 && k == 3) v = 0.0;
         a.diag[cglob * kDiag + k] = v;
+    };
+    double *cta = reinterpret_cast<double *>(static_cast<unsigned char *>(a.fin) + a.fin_off) + c * C * kDiag;   // [C][kDiag]
+    if (tid < kDiag) {
+        double v = red[0][tid];
+        for (int w = 1; w < kFinThreads / 32; ++w) v = merge(tid, v, red[w][tid]);
+        if (C == 1) finish(tid, v);
+        else cta[rank * kDiag + tid] = v;
     }
-    cl.sync();                               // no CTA leaves before rank 0 has read its sums
+    if (C == 1) return;
+    // the CTA that arrives last sums the cell's CTAs in order, and leaves the arrival count at zero
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        int *count = static_cast<int *>(a.fin) + c;
+        last = atomicAdd(count, 1) == C - 1;
+        if (last) *count = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (C <= 8) {
+        if (tid < kDiag) {
+            double v = __ldcg(cta + tid);
+            for (int r = 1; r < C; ++r) v = merge(tid, v, __ldcg(cta + r * kDiag + tid));
+            finish(tid, v);
+        }
+        return;
+    }
+    for (int k = warp; k < kDiag; k += kFinThreads / 32) {
+        double v = k < 7 ? 0.0 : k == 8 ? -1.0e300 : 1.0e300;
+        for (int r = lane; r < C; r += 32) v = merge(k, v, __ldcg(cta + r * kDiag + k));
+#pragma unroll
+        for (int sh = 16; sh > 0; sh >>= 1) v = merge(k, v, __shfl_xor_sync(0xffffffffu, v, sh));
+        if (lane == 0) finish(k, v);
+    }
 }
 
 template <typename T, int D>
 cudaError_t finish_td(int N, const CollideArgs &a, cudaStream_t s)
 {
-    // CTAs per cell: about four vectors a thread, at most 8 (a portable cluster)
-    const int64_t nv = (int64_t)(D == 3 ? N * N : N) * N / FinVec<T>::W;
-    int C = 1;
-    while (C < 8 && nv > (int64_t)C * kFinThreads * 4) C *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.ncells * C), 1, 1);
-    cfg.blockDim = dim3(kFinThreads, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, finish_kernel<T, D>, a, N);
+    finish_kernel<T, D><<<(unsigned)(a.ncells * a.fin_ctas), kFinThreads, 0, s>>>(a, N);
+    return cudaGetLastError();
 }
 
 }  // namespace
+
+// CTAs per cell of the finishing launch: rows enough for a pass of every thread, at most four CTAs per
+// SM in all (one where the cells alone are more)
+int split_finish_ctas(int prec, int d, int N, int64_t n, int sms)
+{
+    const int W = prec == 0 ? 4 : d == 3 ? 2 : 1, rows = d == 3 ? N * N : N;
+    const int64_t most = std::max<int64_t>(1, (int64_t)4 * sms / std::max<int64_t>(n, 1));
+    const int rpc = (int)std::max<int64_t>((kFinThreads * W + N - 1) / N, (rows + most - 1) / most);
+    return (rows + rpc - 1) / rpc;
+}
 
 // loads the finishing kernel (a plan-time call: a first launch under capture could not)
 cudaError_t split_finish_setup(int prec, int d)
