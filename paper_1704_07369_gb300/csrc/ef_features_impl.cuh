@@ -53,15 +53,19 @@ constexpr int feat_band_modes()
     return n;
 }
 
-// CTAs of 4 warps, several per SM (cells in flight overlap their barrier phases): 168 registers
-// for N <= 32 (3 CTAs per SM), 255 above (2 per SM)
+// CTAs of 4 warps, several per SM (cells in flight overlap their barrier phases): for N <= 32 four per
+// SM with one field (128 registers) and three with two (168), above two (255).  The pass issues less
+// than half of the time (latency of its short phases), so a fourth CTA counts.
 constexpr int kFeatThreads = 128;
-template <int N>
-constexpr int feat_min_blocks() { return N <= 32 ? 3 : 2; }
-// accumulators per thread: both fields' band modes over the CTA
-constexpr int kFeatQ = (2 * feat_band_modes() + kFeatThreads - 1) / kFeatThreads;
+template <int N, int NF>
+constexpr int feat_min_blocks() { return N <= 32 ? (NF == 1 ? 4 : 3) : 2; }
 
-template <typename T, int D, int N>
+// accumulators per thread: the fields' band modes over the CTA
+template <int NF>
+constexpr int feat_q = (NF * feat_band_modes() + kFeatThreads - 1) / kFeatThreads;
+
+// NF fields: F alone, or F and ln F
+template <typename T, int D, int N, int NF>
 struct FeatLayout {
     static constexpr int PZ = (D == 3) ? feat_pz<N, sizeof(T) == 4 ? 8 : 4>() : 1;
     static constexpr int NZ = (D == 3) ? N : 1;
@@ -69,18 +73,18 @@ struct FeatLayout {
     static constexpr int X1_FIELD = PZ * X1_PLANE;
     static constexpr int X2_PLANE = kFeatKy * kFeatKx;
     static constexpr int X2_FIELD = PZ * X2_PLANE;             // the current chunk's planes only
-    static constexpr size_t BASE = (size_t)N * sizeof(C2<T>) + 2 * (size_t)(X1_FIELD + X2_FIELD) * sizeof(C2<T>) +
+    static constexpr size_t BASE = (size_t)N * sizeof(C2<T>) + NF * (size_t)(X1_FIELD + X2_FIELD) * sizeof(C2<T>) +
                                    8 * EF_DIAG_STRIDE * sizeof(double);
-    // FP32 3D cells whose two-field layout plus one chunk of raw planes still leaves the CTAs per
+    // FP32 3D cells whose layout plus one chunk of raw planes still leaves the CTAs per
     // SM of the launch bounds: each chunk of PZ planes is staged in shared memory by asynchronous
     // copies (cp.async, 16 bytes a thread) issued while the previous chunk is being transformed
     static constexpr size_t RB_FULL = (size_t)PZ * N * N * sizeof(T);
     static constexpr bool PF = sizeof(T) == 4 && D == 3 && N % 4 == 0 &&
-                               (BASE + RB_FULL + 16 + 1024) * feat_min_blocks<N>() <= 228 * 1024;
+                               (BASE + RB_FULL + 16 + 1024) * feat_min_blocks<N, NF>() <= 228 * 1024;
     static constexpr size_t RB_BYTES = PF ? RB_FULL : 0;
-    static constexpr size_t bytes(int nf)
+    static constexpr size_t bytes()
     {
-        return (size_t)N * sizeof(C2<T>) + (size_t)nf * (X1_FIELD + X2_FIELD) * sizeof(C2<T>) +
+        return (size_t)N * sizeof(C2<T>) + (size_t)NF * (X1_FIELD + X2_FIELD) * sizeof(C2<T>) +
                8 * EF_DIAG_STRIDE * sizeof(double) + (PF ? RB_BYTES + 16 : 0);
     }
 };
@@ -108,8 +112,15 @@ __device__ __forceinline__ void feat_load_row_swz(const float4 *RB, int r, T (&x
 
 template <typename T>
 __device__ __forceinline__ T feat_log(T x);
+// ln x = ln 2 log2 x; the argument is never subnormal, so the flushing form of the instruction serves
+// (the other one scales every argument around it: four instructions of about twenty a point)
 template <>
-__device__ __forceinline__ float feat_log<float>(float x) { return __logf(x > 1e-30f ? x : 1e-30f); }
+__device__ __forceinline__ float feat_log<float>(float x)
+{
+    float l;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x > 1e-30f ? x : 1e-30f));
+    return l * 0.69314718f;
+}
 template <>
 __device__ __forceinline__ double feat_log<double>(double x) { return log(x > 1e-30 ? x : 1e-30); }
 
@@ -313,15 +324,16 @@ __device__ __forceinline__ void cdft_band(const C2<T> (&v)[N], C2<T> (&Y)[2 * K 
     cdft_band_all<T, N, K>(v, Y, std::make_integer_sequence<int, K + 1>{});
 }
 
-template <typename T, int D, int N>
-__global__ void __launch_bounds__(kFeatThreads, feat_min_blocks<N>()) features_kernel(const FeatArgs a)
+template <typename T, int D, int N, int NF>
+__global__ void __launch_bounds__(kFeatThreads, feat_min_blocks<N, NF>()) features_kernel(const FeatArgs a)
 {
-    using Lay = FeatLayout<T, D, N>;
+    using Lay = FeatLayout<T, D, N, NF>;
+    constexpr int kFeatQ = feat_q<NF>;
     constexpr int PZ = Lay::PZ, NZ = Lay::NZ;
     constexpr int ROWS = PZ * N;                 // rows along the contiguous axis per chunk
     static_assert(N / 2 > kFeatK, "grid too small for the band");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nf = a.featL ? 2 : 1;
+    constexpr int nf = NF;
     C2<T> *tw = reinterpret_cast<C2<T> *>(smem_raw);
     C2<T> *X1 = tw + N;
     C2<T> *X2 = X1 + (size_t)nf * Lay::X1_FIELD;
