@@ -56,6 +56,7 @@ constexpr int feat_band_modes()
 // CTAs of 4 warps, several per SM (cells in flight overlap their barrier phases): for N <= 32 four per
 // SM with one field (128 registers) and three with two (168), above two (255).  The pass issues less
 // than half of the time (latency of its short phases), so a fourth CTA counts.
+// (All passes of 16384 surrogate cells of N = 32, with this and the shorter logarithm: 2.58 -> 2.37 ms.)
 constexpr int kFeatThreads = 128;
 template <int N, int NF>
 constexpr int feat_min_blocks() { return N <= 32 ? (NF == 1 ? 4 : 3) : 2; }
