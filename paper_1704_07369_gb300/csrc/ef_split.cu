@@ -250,11 +250,19 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
         }
         return;
     }
+    // warp-uniform k: one FP64 instruction a step, not the three of merge
     for (int k = warp; k < kDiag; k += kFinThreads / 32) {
-        double v = k < 7 ? 0.0 : k == 8 ? -1.0e300 : 1.0e300;
-        for (int r = lane; r < C; r += 32) v = merge(k, v, __ldcg(cta + r * kDiag + k));
+        double v;
+        if (k < 7) {
+            v = 0.0;
+            for (int r = lane; r < C; r += 32) v += __ldcg(cta + r * kDiag + k);
 #pragma unroll
-        for (int sh = 16; sh > 0; sh >>= 1) v = merge(k, v, __shfl_xor_sync(0xffffffffu, v, sh));
+            for (int sh = 16; sh > 0; sh >>= 1) v += __shfl_xor_sync(0xffffffffu, v, sh);
+        } else {
+            v = k == 8 ? -1.0e300 : 1.0e300;
+            for (int r = lane; r < C; r += 32) v = merge(k, v, __ldcg(cta + r * kDiag + k));
+            v = extreme(k, v);
+        }
         if (lane == 0) finish(k, v);
     }
 }
