@@ -96,7 +96,7 @@ enum Epilogue { EPI_FWD = 0, EPI_DW = 1, EPI_DA = 2 };
 // in K order by one accumulator chain, whatever the tile or stage count.  Results leave through
 // shared memory as 16-byte pieces of rows, for the transposed copies too; the element-wise passes that
 // followed a product (fold of the halves, relu mask, row sums) are its epilogue.  Loss and gradients of
-// a 1024-row batch (928 - 512 x 3 - 926): 300 -> 176 us, 27 launches -> 15.
+// a 1024-row batch (928 - 512 x 3 - 926): 300 -> 169 us, 27 launches -> 15.
 template <int MODE>
 __global__ void __launch_bounds__(128) gemm_sync_kernel(const GemmArgs g)
 {
@@ -133,7 +133,10 @@ __global__ void __launch_bounds__(128) gemm_sync_kernel(const GemmArgs g)
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.f;
-    float rowsum = 0.f;                                        // EPI_DW: row tid of A (tid < 64)
+    // EPI_DW: sums of A's rows, two threads a row, as an unevaluated pair (Knuth's TwoSum): the 64 values
+    // of a K block in a tree, the blocks without rounding.  (320 sums of 16384 values of one sign over
+    // eight binary orders: largest relative error 7e-7 with one FP32 chain, 4e-8 so.)
+    [[maybe_unused]] float rs_hi = 0.f, rs_lo = 0.f;
 
     for (int kt = 0; kt < NSTAGE - 1; ++kt) load_tile(kt);
     for (int kt = 0; kt < nk; ++kt) {
@@ -141,16 +144,25 @@ __global__ void __launch_bounds__(128) gemm_sync_kernel(const GemmArgs g)
         __syncthreads();                                       // block kt has landed; block kt - 1 is read
         load_tile(kt + NSTAGE - 1);
         const bf16 *a = sA + (kt % NSTAGE) * BM * LDS, *b = sB + (kt % NSTAGE) * BN * LDS;
-        if (MODE == EPI_DW && blockIdx.x == 0 && g.db && tid < BM) {
-            float t = 0.f;
+        if constexpr (MODE == EPI_DW) {
+            if (blockIdx.x == 0 && g.db) {
+                float t[8] = {};
 #pragma unroll
-            for (int k8 = 0; k8 < BK; k8 += 8) {
-                const uint4 w = *reinterpret_cast<const uint4 *>(a + tid * LDS + k8);
-                const bf16 *e = reinterpret_cast<const bf16 *>(&w);
+                for (int k8 = 0; k8 < BK / 2; k8 += 8) {
+                    const uint4 w = *reinterpret_cast<const uint4 *>(a + (tid >> 1) * LDS + (tid & 1) * (BK / 2) + k8);
+                    const bf16 *e = reinterpret_cast<const bf16 *>(&w);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) t += __bfloat162float(e[j]);
+                    for (int j = 0; j < 8; ++j) t[j] += __bfloat162float(e[j]);
+                }
+#pragma unroll
+                for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+                    for (int j = 0; j < h; ++j) t[j] += t[j + h];
+                const float b = t[0] + __shfl_xor_sync(0xffffffffu, t[0], 1);
+                const float sum = rs_hi + b, bb = sum - rs_hi;
+                rs_lo += (rs_hi - (sum - bb)) + (b - bb);
+                rs_hi = sum;
             }
-            rowsum += t;
         }
 #pragma unroll
         for (int kk = 0; kk < BK; kk += 16) {
@@ -205,7 +217,8 @@ __global__ void __launch_bounds__(128) gemm_sync_kernel(const GemmArgs g)
             }
             __syncthreads();
         }
-        if (blockIdx.x == 0 && g.db && tid < BM) g.db[m0 + tid] = rowsum;
+        // an overflowed sum stays infinite (its low part is a NaN)
+        if (blockIdx.x == 0 && g.db && !(tid & 1)) g.db[m0 + (tid >> 1)] = isinf(rs_hi) ? rs_hi : rs_hi + rs_lo;
         return;
     } else {
         bf16 *st = reinterpret_cast<bf16 *>(sync_raw);         // [hi, hi^T, lo, lo^T][64][LDS]
