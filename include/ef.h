@@ -111,9 +111,10 @@ ef_status ef_collide(ef_plan_t plan, const void *F_dev, void *Q_dev, int64_t nce
 
 /* nsteps forward Euler steps F <- F + dt Q^sigma[F], in place.  If diag_dev is not null it
  * receives nsteps * ncells * EF_DIAG_STRIDE doubles ([step][cell][k], moments of F before each
- * step, entropy production of that step, max nu and the min of the updated F); a step whose
- * updated F has a negative value sets EF_ERR_POSITIVITY in the status word (positivity holds when
- * dt max nu <= 1, proof of Theorem 1). */
+ * step, entropy production of that step, max nu and the min of the updated F).  EF_ERR_POSITIVITY is
+ * set in the status word when the updated F of a cell has a negative value and dt max nu > 1 in that
+ * cell (positivity holds when dt max nu <= 1, proof of Theorem 1: a value below zero is rounding, or
+ * was in F, then).  The report does not depend on how many cells the call has. */
 ef_status ef_euler_step(ef_plan_t plan, void *F_dev, double dt, int nsteps, double *diag_dev,
                         int64_t ncells, ef_stream_t stream);
 

@@ -82,6 +82,11 @@ struct Sync {
     {
         if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     }
+    // war_arrive() that also publishes prior (distributed) shared-memory writes
+    __device__ __forceinline__ void release_arrive()
+    {
+        if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
     __device__ __forceinline__ void war_wait()
     {
         if (C == 1) __syncthreads();
@@ -300,13 +305,22 @@ __device__ __forceinline__ void store_row(T *dst, const T (&x)[N])
     }
 }
 
+// Positivity: an Euler step sets EF_ERR_POSITIVITY where a cell has an updated value below zero and
+// dt nu > 1 somewhere (dt max nu <= 1 keeps F >= 0, so there a value below zero is rounding).  Both are
+// properties of the whole cell, so that the report does not depend on how the cell is spread over CTAs.
+// Paired op lists know nu first: a CTA that sees dt nu > 1 tells every CTA of the cluster (flag is the
+// same variable of each), which read it in the last op, behind a release / acquire barrier.
+__device__ __forceinline__ void flag_cluster(cg::cluster_group &cl, int C, int *flag)
+{
+    if (atomicExch(flag, 1) == 0)
+        for (int r = 0; r < C; ++r) *cl.map_shared_rank(flag, r) = 1;
+}
+
 // Final output of one real row: Q = q, written as Q (collide) or F + dt Q (Euler), with the
-// non-finite / positivity status checks and the diagnostic sums of the row.  nu (nullable) gives
-// the point-wise collision frequency for the positivity test; otherwise nu_big says whether
-// dt nu > 1 anywhere in this CTA's rows.
+// non-finite status check and the diagnostic sums of the row.  Returns whether an updated value
+// of an Euler step is below zero.
 template <typename T, int D, int N, typename DG>
-__device__ __forceinline__ void emit_row(const CollideArgs &a, const T (&fr)[N], T *Orow, T (&q)[N], const T *nu,
-                                         bool nu_big, int64_t grow, DG &dg)
+__device__ __forceinline__ bool emit_row(const CollideArgs &a, const T (&fr)[N], T *Orow, T (&q)[N], int64_t grow, DG &dg)
 {
     constexpr int N1 = (D == 3) ? N : 1;
     const int jz = (int)(grow / N1) - N / 2;
@@ -321,8 +335,7 @@ __device__ __forceinline__ void emit_row(const CollideArgs &a, const T (&fr)[N],
         T outv;
         if (a.out_mode == OUT_EULER) {
             outv = f + T(a.dt) * qv;
-            const bool big = nu ? (T(a.dt) * nu[n] > T(1)) : nu_big;
-            if (outv < T(0) && big) neg = true;
+            if (outv < T(0)) neg = true;
         } else {
             outv = qv;
         }
@@ -344,8 +357,18 @@ __device__ __forceinline__ void emit_row(const CollideArgs &a, const T (&fr)[N],
     }
     store_row<T, N>(Orow, q);
     if (bad) record_status(a.status, 7);     // EF_ERR_NOT_FINITE
-    if (neg) record_status(a.status, 6);     // EF_ERR_POSITIVITY
     if (a.diag) dg.template add_row<D, T>(s_m, s_mx, s_e2, s_eta, s_prod, jz, jy, mn_f, mn_out);
+    return neg;
+}
+
+// The same of a single-slab list, where nu comes last: each thread's findings (1: a value below zero,
+// 2: dt nu > 1) meet in rank 0's flag.
+__device__ __forceinline__ void meet_positivity(const CollideArgs &a, unsigned found, cg::cluster_group &cl, Sync &bar,
+                                                int rank, int tid, int *flag)
+{
+    if (found) atomicOr(cl.map_shared_rank(flag, 0), (int)found);
+    bar.full();
+    if (rank == 0 && tid == 0 && *flag == 3) record_status(a.status, 6);     // EF_ERR_POSITIVITY
 }
 
 // Distributed shared memory through explicit shared::cluster addresses: mapa turns this CTA's
@@ -646,6 +669,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
         Diag dg;
         dg.reset();
         bool have_g = false;                // split: this part's G is already set
+        unsigned found = 0;                 // single-slab Euler step: what this thread's rows show (meet_positivity)
 
         for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
@@ -721,7 +745,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                         const int64_t grow = (int64_t)rank * rows + r;
                         T fr[N];
                         load_row<T, N>(F + grow * N, fr);
-                        emit_row<T, D, N>(a, fr, Out + grow * N, qv, nullptr, big, grow, dg);
+                        if (emit_row<T, D, N>(a, fr, Out + grow * N, qv, grow, dg) && big) record_status(a.status, 6);
                     }
                 }
             } else {
@@ -779,7 +803,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                             }
                             dg.max_nu = fmax(dg.max_nu, (double)mx);
                         }
-                        if (big && a.out_mode == OUT_EULER) *s_nubig = 1;
+                        if (big && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
                     } break;
                     default: {  // OP_LOSS (single mode, last): Q = G - F nu; output; diagnostics
 #pragma unroll
@@ -797,9 +821,10 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
                             for (int n = 0; n < N; ++n) {
                                 qv[n] = Gr[n * rows] - fr[n] * nu[n];
                                 mx = nu[n] > mx ? nu[n] : mx;
+                                if (T(a.dt) * nu[n] > T(1)) found |= 2;
                             }
                             dg.max_nu = fmax(dg.max_nu, (double)mx);
-                            emit_row<T, D, N>(a, fr, Out + grow * N, qv, nu, false, grow, dg);
+                            if (emit_row<T, D, N>(a, fr, Out + grow * N, qv, grow, dg)) found |= 1;
                         }
                     } break;
                     }
@@ -822,6 +847,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads,
             continue;
         }
 
+        if (!a.paired && a.out_mode == OUT_EULER) meet_positivity(a, found, cl, bar, rank, tid, s_nubig);
         // ---------------- per-cell FP64 reduction of the diagnostics
         if (a.diag) diag_reduce_f64<D>(a, dg, part, lane, tid, nt, rank, C, bar, cl, cglob);
     }

@@ -124,8 +124,8 @@ __device__ __forceinline__ void quad_store(double *dst, const double (&x)[M])
 
 // emit_row for a lane's block of M values starting at x0
 template <int D, int N>
-__device__ __forceinline__ void quad_emit(const CollideArgs &a, const double (&fr)[N / 4], double *O, double (&q)[N / 4],
-                                          const double *nu, bool nu_big, int64_t grow, int x0, bool live, Diag &dg)
+__device__ __forceinline__ bool quad_emit(const CollideArgs &a, const double (&fr)[N / 4], double *O, double (&q)[N / 4],
+                                          int64_t grow, int x0, bool live, Diag &dg)
 {
     constexpr int N1 = (D == 3) ? N : 1, M = N / 4;
     const int jz = (int)(grow / N1) - N / 2;
@@ -139,8 +139,7 @@ __device__ __forceinline__ void quad_emit(const CollideArgs &a, const double (&f
         double outv = qv;
         if (a.out_mode == OUT_EULER) {
             outv = f + a.dt * qv;
-            const bool big = nu ? (a.dt * nu[n] > 1.0) : nu_big;
-            if (outv < 0.0 && big) neg = true;
+            if (outv < 0.0) neg = true;
         }
         q[n] = outv;
         if (!isfinite(outv)) bad = true;
@@ -158,11 +157,11 @@ __device__ __forceinline__ void quad_emit(const CollideArgs &a, const double (&f
             mn_out = outv < mn_out ? outv : mn_out;
         }
     }
-    if (!live) return;
+    if (!live) return false;
     quad_store<M>(O, q);
     if (bad) record_status(a.status, 7);     // EF_ERR_NOT_FINITE
-    if (neg) record_status(a.status, 6);     // EF_ERR_POSITIVITY
     if (a.diag) dg.template add_row<D, double>(s_m, s_mx, s_e2, s_eta, s_prod, jz, jy, mn_f, mn_out);
+    return neg;
 }
 
 template <int D, int N>
@@ -342,6 +341,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
         Diag dg;
         dg.reset();
         bool have_g = false;                        // single mode, split: G already set in this part
+        unsigned found = 0;                         // single-slab Euler step: what this thread's rows show
 
         for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
 #pragma unroll
                         for (int n = 0; n < M; ++n) qv[n] = Gr[n * rows] + z[n].x * z[n].y;
                         quad_load<M>(F + grow * N + xb, fr);
-                        quad_emit<D, N>(a, fr, Out + grow * N + xb, qv, nullptr, big, grow, xb, has, dg);
+                        if (quad_emit<D, N>(a, fr, Out + grow * N + xb, qv, grow, xb, has, dg) && big) record_status(a.status, 6);
                     }
                 }
                 have_g = true;
@@ -465,12 +465,13 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
                                 if (has) {
 #pragma unroll
                                     for (int n = 0; n < M; ++n) Gr[n * rows] = -fr[n] * nu[n];
-                                    if (big && a.out_mode == OUT_EULER) *s_nubig = 1;
+                                    if (big && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
                                 }
                             } else {
 #pragma unroll
                                 for (int n = 0; n < M; ++n) qv[n] = Gr[n * rows] - fr[n] * nu[n];
-                                quad_emit<D, N>(a, fr, Out + grow * N + xb, qv, nu, false, grow, xb, has, dg);
+                                if (has && big) found |= 2;
+                                if (quad_emit<D, N>(a, fr, Out + grow * N + xb, qv, grow, xb, has, dg)) found |= 1;
                             }
                         }
                     }
@@ -497,6 +498,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
             continue;
         }
 
+        if (!a.paired && a.out_mode == OUT_EULER) meet_positivity(a, found, cl, bar, rank, tid, s_nubig);
         // ---------------- per-cell FP64 reduction of the diagnostics
         if (a.diag) diag_reduce_f64<D>(a, dg, part, lane, tid, nt, rank, C, bar, cl, cglob);
     }

@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                             const int64_t grow = (int64_t)rank * rows + r;
                             T fr[N];
                             load_row<T, N>(F + grow * N, fr);
-                            emit_row<T, D, N>(a, fr, Out + grow * N, qv, nullptr, big, grow, dg);
+                            if (emit_row<T, D, N>(a, fr, Out + grow * N, qv, grow, dg) && big) record_status(a.status, 6);
                         }
                     }
                 } else {
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                             const int64_t grow = (int64_t)rank * rows + r;
                             T fr[N];
                             load_row<T, N>(F + grow * N, fr);
-                            emit_row<T, D, N>(a, fr, Out + grow * N, qv, nullptr, big, grow, dg);
+                            if (emit_row<T, D, N>(a, fr, Out + grow * N, qv, grow, dg) && big) record_status(a.status, 6);
                         }
                     }
                 }
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         mxt = mx > mxt ? mx : mxt;
                     }
                 }
-                if (bigt && a.out_mode == OUT_EULER) *s_nubig = 1;
+                if (bigt && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
 #pragma unroll
                 for (int o2 = 16; o2 > 0; o2 >>= 1) {
                     const T u = __shfl_xor_sync(wmask, mxt, o2);
@@ -647,8 +647,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                 }
                 if (lane == 0) s_maxnu[tid >> 5] = mxt;
             }
-            // write-after-read: the next op's scatter waits for this arrival
-            bar.war_arrive();
+            // write-after-read: the next op's scatter waits for this arrival.  With st.async no other
+            // barrier orders the loss op's flag of the cell, so that arrival releases it
+            if (ASYNC && !pair) bar.release_arrive();
+            else bar.war_arrive();
             if (o + 1 == o1) bar.war_wait();
         }
 

@@ -102,8 +102,8 @@ __device__ __forceinline__ void tm_c2r_load(const C2<float> *R0, int y0, const C
 // Output of one half row [x0, x0 + N/2): Q = q, written as Q (collide) or F + dt Q (Euler), with
 // the status checks and the half row's share of the diagnostic sums (the same sums as emit_row).
 template <int N>
-__device__ __forceinline__ void tm_emit_half(const CollideArgs &a, const float (&fr)[N / 2], float *Ohalf, float (&q)[N / 2],
-                                             bool nu_big, int64_t grow, int x0, DiagF &dg)
+__device__ __forceinline__ bool tm_emit_half(const CollideArgs &a, const float (&fr)[N / 2], float *Ohalf, float (&q)[N / 2],
+                                             int64_t grow, int x0, DiagF &dg)
 {
     constexpr int NH = N / 2;
     const int jz = (int)(grow / N) - N / 2;
@@ -118,7 +118,7 @@ __device__ __forceinline__ void tm_emit_half(const CollideArgs &a, const float (
         float outv;
         if (a.out_mode == OUT_EULER) {
             outv = f + float(a.dt) * qv;
-            if (outv < 0.f && nu_big) neg = true;
+            if (outv < 0.f) neg = true;
         } else {
             outv = qv;
         }
@@ -140,8 +140,8 @@ __device__ __forceinline__ void tm_emit_half(const CollideArgs &a, const float (
     }
     store_row<float, NH>(Ohalf, q);
     if (bad) record_status(a.status, 7);     // EF_ERR_NOT_FINITE
-    if (neg) record_status(a.status, 6);     // EF_ERR_POSITIVITY
     if (a.diag) dg.template add_row<3, float>(s_m, s_mx, s_e2, s_eta, s_prod, jz, jy, mn_f, mn_out);
+    return neg;
 }
 
 // RPT: rows per team (G of RPT half rows per lane in registers; teams = rows / RPT, threads = 2
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(LB, MINB) collide_kernel_tm(const CollideArgs 
                         const int64_t grow = (int64_t)rank * rows + r;
                         T fr[NH];
                         load_row<T, NH>(F + grow * N + s * NH, fr);
-                        tm_emit_half<N>(a, fr, Out + grow * N + s * NH, qv, big, grow, s * NH, dg);
+                        if (tm_emit_half<N>(a, fr, Out + grow * N + s * NH, qv, grow, s * NH, dg) && big) record_status(a.status, 6);
                     }
                 }
             } else {
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(LB, MINB) collide_kernel_tm(const CollideArgs 
                     }
                     mxt = mx > mxt ? mx : mxt;
                 }
-                if (bigt && a.out_mode == OUT_EULER) *s_nubig = 1;
+                if (bigt && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
 #pragma unroll
                 for (int o2 = 16; o2 > 0; o2 >>= 1) {
                     const T u = __shfl_xor_sync(wmask, mxt, o2);
