@@ -95,7 +95,7 @@ template <int N>
 __host__ __device__ constexpr size_t rg_smem_bytes(int planes, int npc, bool g_shared)
 {
     return (size_t)2 * planes * rg_plane_stride<N>() * 8 + (size_t)N * npc * 8 + (g_shared ? (size_t)planes * N * N * 4 : 0) +
-           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float) + N * sizeof(uint2) + 8;
+           (32 + 1) * kDiag * sizeof(double) + 16 + 32 * sizeof(float) + N * sizeof(uint2) + 16;
 }
 
 // lanes of the calling thread's warp that exist: a block whose size is not a multiple of 32 has a
@@ -127,8 +127,8 @@ __device__ __forceinline__ void st_async(uint32_t a, C2<float> v, uint32_t bar)
                  : "memory");
 }
 
-// Wait for one phase of the CTA's slab mbarrier; gives up after about a second of device time (false).
-__device__ __forceinline__ bool slab_wait(uint32_t bar, uint32_t parity)
+// Wait for one phase of the CTA's slab mbarrier; gives up after limit nanoseconds of device time (false).
+__device__ __forceinline__ bool slab_wait(uint32_t bar, uint32_t parity, long long limit)
 {
     uint64_t t0 = 0;
     for (int it = 0;; ++it) {
@@ -140,9 +140,22 @@ __device__ __forceinline__ bool slab_wait(uint32_t bar, uint32_t parity)
             uint64_t t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
             if (t0 == 0) t0 = t;
-            else if (t - t0 > 1000000000ull) return false;
+            else if (t - t0 > (uint64_t)limit) return false;
         }
     }
+}
+
+// A wait that gave up: waits once more (bounded too) for the stores on their way to this CTA, so that none
+// lands after its exit, and leaves the op's number with every CTA of the cluster.  The barrier at the end of
+// the op makes it known to all of them before the next one; a number, not a flag, so that CTAs that compare
+// with the op they have just finished agree even while a later op's failure is being written.
+static __device__ __noinline__ void slab_fail(uint32_t bar, uint32_t parity, long long limit, uint32_t s_fail, uint32_t op, int C, int *status)
+{
+    slab_wait(bar, parity, limit);
+    record_status(status, 5);               // EF_ERR_TIMEOUT
+    for (int r = 0; r < C; ++r)
+        asm volatile("red.relaxed.cluster.shared::cluster.min.u32 [%0], %1;" ::"r"(cluster_map(s_fail, r)), "r"(op) : "memory");
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
 }
 
 // the whole pencil, one 8-byte store per plane (zt: plane address and its owner's mbarrier).  8-byte
@@ -346,7 +359,12 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
     const uint32_t base0 = smem_u32addr(Is0), slab1 = (uint32_t)((size_t)P * NPP * sizeof(C2<T>));
     // the mbarrier of this CTA's slabs: one arrival (the expected bytes) and the bytes themselves per op
     const uint32_t mbar = smem_u32addr(s_zt + N);
-    uint32_t phase = 0;
+    // ASYNC: the op in which a slab wait of the cluster gave up (slab_fail), the ops done so far and whether
+    // it is one of them.  From there on the cluster exchanges nothing more: its cells' outputs become NaN.
+    volatile uint32_t *s_fail = reinterpret_cast<volatile uint32_t *>(s_zt + N + 1);
+    uint32_t nop = 0;
+    bool failed = false;
+    if (ASYNC && tid == 0) *s_fail = 0xffffffffu;
     for (int z = tid; z < N; z += nt)
         s_zt[z] = make_uint2(cluster_map(base0 + (uint32_t)((z % P) * NPP * sizeof(C2<T>)), z / P), cluster_map(mbar, z / P));
     if (ASYNC && tid == 0) {
@@ -385,6 +403,16 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
         const T *F = reinterpret_cast<const T *>(a.F) + coff;
         T *Out = reinterpret_cast<T *>(a.Q) + coff;
         T *pnu = reinterpret_cast<T *>(a.part) + (c * (S + 1) + S) * CELL;       // split: the cell's nu
+        auto give_nan = [&]() {                     // this CTA's rows of the item's output
+            __syncthreads();                        // behind what other threads stored there
+            T *dst = (S > 1 ? reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL : Out) + (int64_t)rank * rows * N;
+            for (int i = tid; i < rows * N; i += nt) dst[i] = __int_as_float(0x7fc00000);
+            if (S == 1 && a.diag && rank == 0 && tid < kDiag) a.diag[cglob * kDiag + tid] = __int_as_float(0x7fc00000);
+        };
+        if (ASYNC && failed) {
+            give_nan();
+            continue;
+        }
         if (tid == 0) *s_nubig = 0;
 
         // ---------------- F1: own rows real -> half complex (k_x < N/2 kept), two rows per item
@@ -476,8 +504,9 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                     __syncwarp(wmask);
                     bar.war_wait();
                     held = false;
+                    if (ASYNC) failed = *s_fail < nop;
                 }
-                if (has) {
+                if (has && !failed) {
                     if constexpr (ASYNC) rg_scatter_async<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_at<N>(ky, kx) * 8));
                     else rg_scatter<N>(v, s_zt, (b ? slab1 : 0u) + (uint32_t)(rg_poff<N>(q & ~1) * 8), q & 1, mask);
                     if (a.prefetch && o + 1 < o1) {
@@ -491,15 +520,19 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                     }
                 }
             }
-            if (held) bar.war_wait();      // warps without an item
+            if (held) {                    // warps without an item
+                bar.war_wait();
+                if (ASYNC) failed = *s_fail < nop;
+            }
             if constexpr (ASYNC) {
+                if (failed) break;         // the whole cluster: nothing of this op has been sent
                 // the peers start the next phase only after this CTA's arrival at the end of the op, so
                 // every byte counts towards the phase that this wait is for
                 if (tid == 0)
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar),
-                                 "r"((uint32_t)((pair ? 2 : 1) * rows * NH * (int)sizeof(C2<T>))) : "memory");
-                if (!slab_wait(mbar, phase)) record_status(a.status, 5);      // EF_ERR_TIMEOUT
-                phase ^= 1;
+                                 "r"((uint32_t)((pair ? 2 : 1) * rows * NH * (int)sizeof(C2<T>) + a.slab_extra)) : "memory");
+                if (!slab_wait(mbar, nop & 1, a.slab_ns)) slab_fail(mbar, nop & 1, a.slab_ns, smem_u32addr((const void *)s_fail), nop, C, a.status);
+                ++nop;
             } else {
                 bar.full();
             }
@@ -651,7 +684,14 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             // barrier orders the loss op's flag of the cell, so that arrival releases it
             if (ASYNC && !pair) bar.release_arrive();
             else bar.war_arrive();
-            if (o + 1 == o1) bar.war_wait();
+            if (o + 1 == o1) {
+                bar.war_wait();
+                if (ASYNC) failed = *s_fail < nop;
+            }
+        }
+        if (ASYNC && failed) {
+            give_nan();
+            continue;
         }
 
         if (S > 1) {                       // this part's gain (zeros from a part with only the loss)

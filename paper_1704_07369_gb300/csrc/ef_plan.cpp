@@ -313,6 +313,7 @@ struct ef_plan_s {
     bool batched = false;
     bool may_split = true;              // launches may split cells into parts (off for plans that run side by side)
     int sms = 1;
+    long long slab_ns = 0;              // > 0: every slab wait of the plan's calls runs out after so long (tests)
     int64_t ncells = 0;
     std::vector<ClassPlan> classes;
     int64_t *d_all_off = nullptr, *d_all_N = nullptr;
@@ -1271,6 +1272,10 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         a.counter = multi ? p->d_counters + ci : nullptr;
         a.prefetch = cp.prefetch;
         a.paired = sh.paired;
+        if (p->slab_ns > 0) {
+            a.slab_ns = p->slab_ns;
+            a.slab_extra = 8;
+        }
         e = launch_shape(ds, cp.N, a, grid, sh, cs);
         if (e != cudaSuccess) return cuda_fail(e, "collide launch");
         if (multi) {
@@ -1288,6 +1293,9 @@ ef_status finish_plan(ef_plan_s *p)
     if (e != cudaSuccess) return cuda_fail(e, "status word");
     e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
     p->slots = std::make_shared<PartSlots>();
+    // EF_SLAB_TIMEOUT_NS: lets the FP32 register kernels' waits of this plan run out after so many
+    // nanoseconds (for tests of what follows: EF_ERR_TIMEOUT and NaN)
+    if (const char *v = std::getenv("EF_SLAB_TIMEOUT_NS")) p->slab_ns = std::atoll(v);
     if (e == cudaSuccess) e = ef::split_finish_setup(p->desc.prec == EF_PREC_F32 ? 0 : 1, p->desc.d);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->split_done, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(e, "plan event");
