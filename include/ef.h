@@ -410,8 +410,9 @@ ef_status ef_plan_set_graph(ef_plan_t plan, int enable);
 
 /* Introspection (host values):  info[0] = d, [1] = number of distinct N, [2] = number of
  * spectral directions (inverse transforms per cell, loss included) of the first class, [3] =
- * cluster size of the first class, [4] = threads per CTA of the first class, [5] = cells (batched
- * plans; 0 otherwise), [6] = precision, [7] = kernel launches per ef_collide. */
+ * cluster size and [4] = threads per CTA of the first class (a uniform plan: of its first shape; a call
+ * may use another one, ef_plan_call_info), [5] = cells (batched plans; 0 otherwise), [6] = precision,
+ * [7] = collide launches per ef_collide, one per class (a split class has a finishing launch besides). */
 ef_status ef_plan_info(ef_plan_t plan, int64_t info[8]);
 
 /* Launch shape of size class i (0 <= i < info[1] of ef_plan_info), host values:
@@ -420,6 +421,15 @@ ef_status ef_plan_info(ef_plan_t plan, int64_t info[8]);
  * global memory, [6] = 1 if the next multiplier slice is prefetched, [7] = autotuned time of one
  * class launch in microseconds (0 when not tuned).  EF_ERR_INVALID_ARG for a bad index. */
 ef_status ef_plan_class_info(ef_plan_t plan, int i, int64_t out[8]);
+
+/* What a call on ncells cells launches for size class i (a batched plan: on its own cells, ncells is
+ * ignored).  A call with fewer cells than the device holds clusters may run each cell's directions as
+ * several parts on as many clusters, whose gains a finishing launch sums; the shape of a uniform plan's
+ * call depends on its cell count.  out[0] = parts per cell (1: not split), [1] = cluster size, [2] = threads
+ * per CTA, [3] = kernel variant, [4] = kernel launches, [5] = clusters of the collide launch, [6..7] = 0.
+ * split = 0: the launch of a call that may not be split.  Host only; nothing is launched.
+ * EF_ERR_INVALID_ARG for a bad index or ncells <= 0 (uniform plans). */
+ef_status ef_plan_call_info(ef_plan_t plan, int i, int64_t ncells, int split, int64_t out[8]);
 
 const char *ef_status_string(ef_status s);
 const char *ef_last_error(void);

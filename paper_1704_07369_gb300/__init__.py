@@ -35,7 +35,7 @@ EF_DIAG_STRIDE = 10
 # every symbol include/ef.h declares
 SYMBOLS = ("ef_plan_create", "ef_plan_create_ex", "ef_plan_create_batched", "ef_plan_destroy",
            "ef_collide", "ef_euler_step", "ef_rk3_step", "ef_moments_entropy", "ef_plan_status",
-           "ef_plan_set_graph", "ef_plan_info", "ef_plan_class_info", "ef_plan_reserve", "ef_collide_noalloc", "ef_kernel_G",
+           "ef_plan_set_graph", "ef_plan_info", "ef_plan_class_info", "ef_plan_call_info", "ef_plan_reserve", "ef_collide_noalloc", "ef_kernel_G",
            "ef_galerkin_create", "ef_galerkin_collide", "ef_galerkin_status", "ef_galerkin_destroy",
            "ef_features", "ef_mlp_create", "ef_mlp_destroy", "ef_mlp_info", "ef_mlp_status", "ef_mlp_params",
            "ef_mlp_forward", "ef_mlp_grad", "ef_mlp_train_step",
@@ -128,6 +128,7 @@ def lib():
         L.ef_plan_set_graph.argtypes = [vp, i32]
         L.ef_plan_info.argtypes = [vp, ctypes.POINTER(i64)]
         L.ef_plan_class_info.argtypes = [vp, i32, ctypes.POINTER(i64)]
+        L.ef_plan_call_info.argtypes = [vp, i32, i64, i32, ctypes.POINTER(i64)]
         L.ef_status_string.restype = ctypes.c_char_p
         L.ef_status_string.argtypes = [i32]
         L.ef_last_error.restype = ctypes.c_char_p
@@ -460,6 +461,13 @@ def ef_plan_class_info(plan, i):
     return dict(zip(keys, list(out)))
 
 
+def ef_plan_call_info(plan, i, ncells, split=1):
+    out = (ctypes.c_int64 * 8)()
+    _check(lib().ef_plan_call_info(plan, int(i), int(ncells), int(split), out))
+    keys = ("parts", "cluster", "threads", "variant", "launches", "clusters")
+    return dict(zip(keys, list(out)))
+
+
 class Plan:
     """Owning wrapper of an ``ef_plan_t``."""
 
@@ -560,6 +568,10 @@ class Plan:
 
     def class_info(self):
         return [ef_plan_class_info(self.handle, i) for i in range(self.info()["classes"])]
+
+    def call_info(self, ncells=0, split=1):
+        """What a call on ncells cells launches, per size class."""
+        return [ef_plan_call_info(self.handle, i, ncells, split) for i in range(self.info()["classes"])]
 
     def _n(self, F, ncells):
         if ncells is not None:

@@ -1849,6 +1849,25 @@ ef_status ef_plan_class_info(ef_plan_t p, int i, int64_t out[8])
     return EF_OK;
 }
 
+ef_status ef_plan_call_info(ef_plan_t p, int i, int64_t ncells, int split, int64_t out[8])
+{
+    if (!p || !out) return fail(EF_ERR_INVALID_ARG, "null plan or output");
+    if (i < 0 || i >= (int)p->classes.size()) return fail(EF_ERR_INVALID_ARG, "class index out of range");
+    if (!p->batched && ncells <= 0) return fail(EF_ERR_INVALID_ARG, "ncells <= 0");
+    ClassPlan &cp = p->classes[i];
+    const int64_t n = p->batched ? cp.ncells : ncells;
+    int S = 1;
+    const Shape &sh = call_shape(p, cp, n, split != 0, S);
+    out[0] = S;
+    out[1] = sh.cluster;
+    out[2] = sh.tpb;
+    out[3] = sh.occ;
+    out[4] = S > 1 ? 2 : 1;
+    out[5] = std::min<int64_t>(n * S, sh.max_clusters);
+    out[6] = out[7] = 0;
+    return EF_OK;
+}
+
 ef_status ef_plan_info(ef_plan_t p, int64_t info[8])
 {
     if (!p || !info) return fail(EF_ERR_INVALID_ARG, "null plan or info");
