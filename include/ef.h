@@ -26,7 +26,19 @@
  *   synchronises the device or blocks the host, except ef_plan_destroy and ef_plan_status(plan, 1);
  *   so the operations can be captured into a CUDA graph.
  * Streams: operations are enqueued on the given CUDA stream (0 = legacy default stream) and return
- *   immediately.  The plan's device must be current on the calling thread.
+ *   immediately.  The plan's device must be current on the calling thread.  A plan may be used on
+ *   several streams: operations whose kernels need its workspaces (FP64, 2D, FP32 3D below N = 16, calls
+ *   that split their cells, ef_rk3_step) wait for the last one that did, on whatever stream.
+ * Captures: such operations captured on one stream of one capture get a workspace of their graph's own
+ *   (four per plan, given back when the graph and its executables are destroyed), so that the graph may be
+ *   replayed beside calls and other graphs.  With all four taken they are captured without splitting cells
+ *   (for a few cells many times slower; ef_plan_call_info, split = 0), and on the calls' workspace: graphs
+ *   of those kinds must then not be replayed beside other operations of the plan.  Neither may graphs of
+ *   ef_rk3_step, whose stage buffers all share.
+ * Reproducibility: the same operation on the same cells, of a plan made alike, gives the same bits where
+ *   it is launched alike.  How a cell's sums are ordered depends on the launch, and that on the number of
+ *   cells in the call (uniform plans), on timings at creation (batched plans; EF_AUTOTUNE_CACHE keeps them)
+ *   and on the workspace a capture found: such results differ by rounding.
  * Errors: every function returns an ef_status; on failure nothing is launched and
  *   ef_last_error() (thread-local) describes why.  Argument checks run before any launch.
  *   Device-side conditions (non-finite values, a positivity violation under an Euler step) are

@@ -259,10 +259,11 @@ struct ClassPlan {
     int64_t pick_n = -1;                // the last choice: cell count, shape, parts
     size_t pick_i = 0;
     int pick_s = 1;
-    void *d_part = nullptr;             // gains of the parts of split launches, kPartSlots workspaces
-    size_t part_bytes = 0;              // of one workspace
-    void *d_fin = nullptr;              // arrivals and diagnostics of the finishing launches, kPartSlots of them
-    size_t fin_off = 0, fin_bytes = 0;  // diagnostics behind the arrivals, bytes of one
+    // kWorkSlots workspaces of each kind that the class needs, *_bytes one of them
+    void *d_part = nullptr;             // gains of the parts of split launches
+    size_t part_bytes = 0;
+    void *d_fin = nullptr;              // arrivals and diagnostics of the finishing launches
+    size_t fin_off = 0, fin_bytes = 0;  // diagnostics behind the arrivals
     size_t smem = 0;
     int max_clusters = 0;
     int ndir = 0, nops = 0;              // op count of the active mode
@@ -273,31 +274,34 @@ struct ClassPlan {
     ef::Op *d_ops_single = nullptr, *d_ops_paired = nullptr;
     int *d_modes = nullptr;              // band modes [nfeat][3] (|k| <= EF_FEATURE_K), feature slot order
     int64_t *d_cell_off = nullptr, *d_cell_id = nullptr;
-    void *d_sg = nullptr;
+    void *d_sg = nullptr;                // S/G accumulators of sg_slots clusters
+    size_t sg_bytes = 0;
     int64_t sg_slots = 0;
-    void *d_fh = nullptr;                // forward-spectrum workspace, fh_slots clusters
+    void *d_fh = nullptr;                // forward spectra of fh_slots clusters
+    size_t fh_bytes = 0;
     int64_t fh_slots = 0;
 };
 
 }  // namespace
 
-// Part workspaces of a plan: 0 for calls, the rest for callers' stream captures.  A graph may be replayed
-// beside anything, so the split calls captured on one stream of one capture take a workspace that no
-// other graph uses, and give it back when the graph and its executables are destroyed (a user object
-// that the graph retains).  With none left a captured call is not split.
-constexpr int kPartSlots = 5;
-struct PartSlots {
-    std::atomic<int> taken[kPartSlots]{};
-    unsigned long long capture[kPartSlots]{};
-    cudaStream_t stream[kPartSlots]{};      // of the capture that holds the workspace
+// Workspaces of a plan (part gains, forward spectra, global accumulators): 0 for calls, the rest for callers'
+// stream captures.  A graph may be replayed beside calls and other graphs, so the calls captured on one
+// stream of one capture take a workspace that no other graph uses, and give it back when the graph and its
+// executables are destroyed (a user object that the graph retains).  With none left a captured call is
+// not split and, where its kernels need a workspace at all, shares workspace 0.
+constexpr int kWorkSlots = 5;
+struct WorkSlots {
+    std::atomic<int> taken[kWorkSlots]{};
+    unsigned long long capture[kWorkSlots]{};
+    cudaStream_t stream[kWorkSlots]{};      // of the capture that holds the workspace
 };
-struct PartLease {
-    std::shared_ptr<PartSlots> slots;
+struct WorkLease {
+    std::shared_ptr<WorkSlots> slots;
     int i;
 };
 void CUDART_CB end_lease(void *p)
 {
-    PartLease *l = static_cast<PartLease *>(p);
+    WorkLease *l = static_cast<WorkLease *>(p);
     l->slots->taken[l->i].store(0);
     delete l;
 }
@@ -330,11 +334,11 @@ struct ef_plan_s {
     double *g_diag = nullptr;
     int g_slot = -1;
     cudaStream_t g_stream = nullptr;
-    // split launches share the part workspace 0: an event behind the last one, which the next waits for
-    // (nothing to wait for on the same stream); captured calls have workspaces 1 .. of their graphs
-    cudaEvent_t split_done = nullptr;
-    bool split_used = false;
-    std::shared_ptr<PartSlots> slots;
+    // calls that use workspace 0 (or the SSP-RK3 buffers): an event behind the last one, which the next waits
+    // for (nothing to wait for on the same stream); captured calls have workspaces 1 .. of their graphs
+    cudaEvent_t work_done = nullptr;
+    bool work_used = false;
+    std::shared_ptr<WorkSlots> slots;
     // SSP-RK3 stage buffers: two batch-sized arrays, grown on demand
     void *d_rk = nullptr;
     size_t rk_bytes = 0;
@@ -377,6 +381,9 @@ cudaError_t launch_for(int prec, int d, int N, const ef::CollideArgs &a, int gri
     return d == 3 ? ef::collide_launch_f64_3d(N, a, grid, tpb, smem, occ, s)
                   : ef::collide_launch_f64_2d(N, a, grid, tpb, smem, occ, s);
 }
+
+// The register kernels keep the forward spectrum in shared memory.
+bool uses_fh(const Desc &ds, const Shape &sh) { return !(ds.prec == EF_PREC_F32 && ds.d == 3 && sh.occ >= 3); }
 
 // One class launch in shape sh, with the finishing launch of a split one behind it.
 cudaError_t launch_shape(const Desc &ds, int N, const ef::CollideArgs &a, int grid, const Shape &sh, cudaStream_t s)
@@ -977,9 +984,9 @@ ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split, int sms)
     return choose_shape(ds, cp, cp.ncells > 0 ? std::min<int64_t>(cp.ncells, 2048) : 0, may_split, sms);
 }
 
-// Workspaces of one class for every cluster that can be resident at once (max_clusters, fixed by
-// the chosen launch shape): the forward-spectrum slots and, for the global-accumulator shapes, the
-// S/G slots.  Called once at plan creation, so that no operation allocates.
+// Workspaces of one class for every cluster that can be resident at once (max_clusters, fixed by the
+// launch shapes): forward spectra, S/G accumulators of the global-accumulator shapes, and the parts of
+// split launches.  Called once at plan creation, so that no operation allocates.
 ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
 {
     const Desc &ds = p->desc;
@@ -987,10 +994,10 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
     const int64_t cell = (int64_t)cp.N * cp.N * (ds.d == 3 ? cp.N : 1);
     std::vector<Shape> used(1, cp.cur);
     if (!p->batched) used.insert(used.end(), cp.shapes.begin(), cp.shapes.end());
-    int64_t clusters = 1, sg_clusters = 0, part_cells = 0, fin_cells = 0;      // fin_cells: of a split launch
+    int64_t part_cells = 0, fin_cells = 0;      // fin_cells: of a split launch
     for (const Shape &sh : used) {
-        clusters = std::max<int64_t>(clusters, sh.max_clusters);
-        if (sh.sg_global) sg_clusters = std::max<int64_t>(sg_clusters, sh.max_clusters);
+        if (uses_fh(ds, sh)) cp.fh_slots = std::max<int64_t>(cp.fh_slots, sh.max_clusters);
+        if (sh.sg_global) cp.sg_slots = std::max<int64_t>(cp.sg_slots, sh.max_clusters);
         // uniform: n cells in S parts, n S at most the resident clusters, and nu: n (S + 1) <= 3/2 of them
         if (!p->batched && max_split(ds, cp, sh, 1) > 1) fin_cells = std::max<int64_t>(fin_cells, sh.max_clusters);
         if (!p->batched && max_split(ds, cp, sh, 1) > 1) part_cells = std::max<int64_t>(part_cells, sh.max_clusters + (sh.max_clusters + 1) / 2);
@@ -999,24 +1006,22 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
         part_cells = cp.ncells * (cp.split + 1);
         fin_cells = cp.ncells;
     }
-    cudaError_t e = cudaMalloc(&cp.d_fh, (size_t)clusters * ef::collide_fh_bytes(ds.prec, ds.d, cp.N));
-    if (e != cudaSuccess) { cp.d_fh = nullptr; return cuda_fail(e, "spectrum workspace"); }
-    cp.fh_slots = clusters;
-    if (sg_clusters) {
-        e = cudaMalloc(&cp.d_sg, (size_t)sg_clusters * 2 * cell * el);
-        if (e != cudaSuccess) { cp.d_sg = nullptr; return cuda_fail(e, "S/G workspace"); }
-        cp.sg_slots = sg_clusters;
-    }
+    auto alloc = [&](void **q, size_t &bytes, size_t need) {
+        bytes = (need + 255) / 256 * 256;
+        if (!bytes) return cudaSuccess;
+        const cudaError_t e = cudaMalloc(q, kWorkSlots * bytes);
+        if (e != cudaSuccess) *q = nullptr;
+        return e;
+    };
+    cudaError_t e = alloc(&cp.d_fh, cp.fh_bytes, (size_t)cp.fh_slots * ef::collide_fh_bytes(ds.prec, ds.d, cp.N));
+    if (e != cudaSuccess) return cuda_fail(e, "spectrum workspace");
+    e = alloc(&cp.d_sg, cp.sg_bytes, (size_t)cp.sg_slots * 2 * cell * el);
+    if (e != cudaSuccess) return cuda_fail(e, "S/G workspace");
     if (part_cells) {
-        cp.part_bytes = (size_t)part_cells * cell * el;
-        cp.part_bytes = (cp.part_bytes + 255) / 256 * 256;
-        e = cudaMalloc(&cp.d_part, kPartSlots * cp.part_bytes);
-        if (e != cudaSuccess) { cp.d_part = nullptr; return cuda_fail(e, "part workspace"); }
+        e = alloc(&cp.d_part, cp.part_bytes, (size_t)part_cells * cell * el);
         cp.fin_off = fin_offset(fin_cells);
-        cp.fin_bytes = cp.fin_off + fin_diag_bytes(fin_cells, p->sms);
-        e = cudaMalloc(&cp.d_fin, kPartSlots * cp.fin_bytes);
-        if (e != cudaSuccess) { cp.d_fin = nullptr; return cuda_fail(e, "part workspace"); }
-        e = cudaMemset(cp.d_fin, 0, kPartSlots * cp.fin_bytes);
+        if (e == cudaSuccess) e = alloc(&cp.d_fin, cp.fin_bytes, cp.fin_off + fin_diag_bytes(fin_cells, p->sms));
+        if (e == cudaSuccess) e = cudaMemset(cp.d_fin, 0, kWorkSlots * cp.fin_bytes);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();      // whatever stream the first call is on
         if (e != cudaSuccess) return cuda_fail(e, "part workspace");
     }
@@ -1028,7 +1033,7 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
 ef_status check_workspaces(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64_t n, int S, int grid_clusters)
 {
     const size_t cell = (size_t)cp.N * cp.N * (ds.d == 3 ? cp.N : 1) * (ds.prec == EF_PREC_F32 ? 4 : 8);
-    if (grid_clusters > cp.fh_slots || (sh.sg_global && grid_clusters > cp.sg_slots) ||
+    if ((uses_fh(ds, sh) && grid_clusters > cp.fh_slots) || (sh.sg_global && grid_clusters > cp.sg_slots) ||
         (S > 1 && (size_t)n * (S + 1) * cell > cp.part_bytes))
         return fail(EF_ERR_INVALID_ARG, "launch exceeds the plan's workspaces");
     return EF_OK;
@@ -1049,7 +1054,7 @@ void destroy_plan(ef_plan_s *p)
         cudaFree(cp.d_part);
         cudaFree(cp.d_fin);
     }
-    if (p->split_done) cudaEventDestroy(p->split_done);
+    if (p->work_done) cudaEventDestroy(p->work_done);
     cudaFree(p->d_all_off);
     cudaFree(p->d_all_N);
     cudaFree(p->d_rk);
@@ -1132,47 +1137,51 @@ const Shape &call_shape(ef_plan_s *p, ClassPlan &cp, int64_t n, bool split, int 
     return cp.shapes[cp.pick_i];
 }
 
-// The part workspace of one operation: slot >= 0, or -1 where its calls are not split.  Calls share
-// workspace 0: each waits for an event behind the last one, whatever stream that was on.  (No
-// cudaStreamGetId: it ends a capture that is under way.)
-struct SplitUse {
+// The workspace of one operation: slot >= 0, or -1 where its launches need none, or a capture finds none
+// left (its calls are not split then).  Calls share workspace 0: each waits for an event behind the last one
+// that used it, whatever stream that was on.  stages: the operation uses the plan's SSP-RK3 buffers, which
+// calls share in the same way.  (No cudaStreamGetId: it ends a capture that is under way.)
+struct WorkUse {
     ef_plan_s *p;
     cudaStream_t s;
     int slot = -1;
-    SplitUse(ef_plan_s *p_, int64_t ncells, cudaStream_t s_) : p(p_), s(s_)
+    bool record = false;
+    WorkUse(ef_plan_s *p_, int64_t ncells, cudaStream_t s_, bool stages = false) : p(p_), s(s_)
     {
-        bool wants = false;
+        bool needs = false;
         for (ClassPlan &cp : p->classes) {
             int S = 1;
             const int64_t n = p->batched ? cp.ncells : ncells;
-            if (n > 0) call_shape(p, cp, n, true, S);
-            wants = wants || S > 1;
+            if (n <= 0) continue;
+            const Shape &sh = call_shape(p, cp, n, true, S);
+            needs = needs || S > 1 || uses_fh(p->desc, sh) || sh.sg_global;
         }
-        if (!wants) return;
-        if (!begin()) cudaGetLastError();
+        if ((needs || stages) && !begin(needs)) cudaGetLastError();
     }
-    bool begin()
+    bool begin(bool needs)
     {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         unsigned long long capture = 0;
         cudaGraph_t graph = nullptr;
         if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
         if (cap == cudaStreamCaptureStatusNone) {
-            if (p->split_used && cudaStreamWaitEvent(s, p->split_done, 0) != cudaSuccess) return false;
-            slot = 0;
+            if (p->work_used && cudaStreamWaitEvent(s, p->work_done, 0) != cudaSuccess) return false;
+            record = true;
+            if (needs) slot = 0;
             return true;
         }
-        if (cap != cudaStreamCaptureStatusActive || capture_info(s, &cap, &capture, &graph) != cudaSuccess) return false;
-        PartSlots &ps = *p->slots;
-        for (int i = 1; i < kPartSlots; ++i)
-            if (ps.taken[i].load() && ps.capture[i] == capture && ps.stream[i] == s) {
+        if (!needs || cap != cudaStreamCaptureStatusActive) return true;
+        if (capture_info(s, &cap, &capture, &graph) != cudaSuccess) return false;
+        WorkSlots &ws = *p->slots;
+        for (int i = 1; i < kWorkSlots; ++i)
+            if (ws.taken[i].load() && ws.capture[i] == capture && ws.stream[i] == s) {
                 slot = i;
                 return true;
             }
-        for (int i = 1; i < kPartSlots; ++i) {
+        for (int i = 1; i < kWorkSlots; ++i) {
             int free_ = 0;
-            if (!ps.taken[i].compare_exchange_strong(free_, 1)) continue;
-            PartLease *l = new PartLease{p->slots, i};
+            if (!ws.taken[i].compare_exchange_strong(free_, 1)) continue;
+            WorkLease *l = new WorkLease{p->slots, i};
             cudaUserObject_t obj = nullptr;
             if (cudaUserObjectCreate(&obj, l, end_lease, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
                 end_lease(l);
@@ -1182,12 +1191,12 @@ struct SplitUse {
                 cudaUserObjectRelease(obj, 1);            // runs end_lease
                 return false;
             }
-            ps.capture[i] = capture;
-            ps.stream[i] = s;
+            ws.capture[i] = capture;
+            ws.stream[i] = s;
             slot = i;
             return true;
         }
-        return false;
+        return true;
     }
     static cudaError_t capture_info(cudaStream_t s, cudaStreamCaptureStatus *cap, unsigned long long *id, cudaGraph_t *graph)
     {
@@ -1197,11 +1206,11 @@ struct SplitUse {
         return cudaStreamGetCaptureInfo_v2(s, cap, id, graph, nullptr, nullptr);
 #endif
     }
-    ~SplitUse()
+    ~WorkUse()
     {
-        if (slot != 0) return;
-        cudaEventRecord(p->split_done, s);
-        p->split_used = true;
+        if (!record) return;
+        cudaEventRecord(p->work_done, s);
+        p->work_used = true;
     }
 };
 
@@ -1254,15 +1263,16 @@ ef_status run(ef_plan_s *p, const void *F, void *Out, int64_t ncells, int mode, 
         a.cluster = sh.cluster;
         a.planes = sh.planes;
         a.sg_global = sh.sg_global;
-        a.sg_ws = cp.d_sg;
+        const size_t ws = slot > 0 ? slot : 0;
+        if (sh.sg_global) a.sg_ws = static_cast<unsigned char *>(cp.d_sg) + ws * cp.sg_bytes;
+        if (uses_fh(ds, sh)) a.fh_ws = static_cast<unsigned char *>(cp.d_fh) + ws * cp.fh_bytes;
         a.nsplit = S;
-        a.part = static_cast<unsigned char *>(cp.d_part) + (slot > 0 ? slot : 0) * cp.part_bytes;
         if (S > 1) {
-            a.fin = static_cast<unsigned char *>(cp.d_fin) + (slot > 0 ? slot : 0) * cp.fin_bytes;
+            a.part = static_cast<unsigned char *>(cp.d_part) + ws * cp.part_bytes;
+            a.fin = static_cast<unsigned char *>(cp.d_fin) + ws * cp.fin_bytes;
             a.fin_off = cp.fin_off;
             a.fin_ctas = ef::split_finish_ctas(ds.prec == EF_PREC_F32 ? 0 : 1, ds.d, cp.N, n, p->sms);
         }
-        a.fh_ws = cp.d_fh;
         a.npc = ef::collide_npc_v(ds.prec, ds.d, cp.N, sh.cluster, sh.occ);
         a.out_mode = mode;
         a.dt = dt;
@@ -1292,12 +1302,12 @@ ef_status finish_plan(ef_plan_s *p)
     cudaError_t e = cudaMalloc((void **)&p->d_status, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "status word");
     e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
-    p->slots = std::make_shared<PartSlots>();
+    p->slots = std::make_shared<WorkSlots>();
     // EF_SLAB_TIMEOUT_NS: lets the FP32 register kernels' waits of this plan run out after so many
     // nanoseconds (for tests of what follows: EF_ERR_TIMEOUT and NaN)
     if (const char *v = std::getenv("EF_SLAB_TIMEOUT_NS")) p->slab_ns = std::atoll(v);
     if (e == cudaSuccess) e = ef::split_finish_setup(p->desc.prec == EF_PREC_F32 ? 0 : 1, p->desc.d);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->split_done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->work_done, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(e, "plan event");
     e = cudaMemset(p->d_status, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "status word");
@@ -1624,7 +1634,7 @@ ef_status ef_collide(ef_plan_t p, const void *F, void *Q, int64_t ncells, ef_str
     if (((uintptr_t)F | (uintptr_t)Q) % 16) return fail(EF_ERR_INVALID_ARG, "F and Q must be 16-byte aligned");
     ef_status st = check_device(p);
     if (st != EF_OK) return st;
-    const SplitUse use(p, ncells, (cudaStream_t)stream);
+    const WorkUse use(p, ncells, (cudaStream_t)stream);
     return step(p, F, Q, ncells, ef::OUT_COLLIDE, 0.0, nullptr, use.slot, (cudaStream_t)stream);
 }
 
@@ -1639,7 +1649,7 @@ ef_status ef_euler_step(ef_plan_t p, void *F, double dt, int nsteps, double *dia
     if ((uintptr_t)F % 16) return fail(EF_ERR_INVALID_ARG, "F must be 16-byte aligned");
     ef_status st = check_device(p);
     if (st != EF_OK) return st;
-    const SplitUse use(p, ncells, (cudaStream_t)stream);
+    const WorkUse use(p, ncells, (cudaStream_t)stream);
     for (int k = 0; k < nsteps; ++k) {
         st = step(p, F, F, ncells, ef::OUT_EULER, dt, diag ? diag + (int64_t)k * ncells * ef::kDiag : nullptr,
                   use.slot, (cudaStream_t)stream);
@@ -1711,7 +1721,7 @@ ef_status ef_rk3_step(ef_plan_t p, void *F, double dt, int nsteps, double *diag,
     void *A = p->d_rk, *B = static_cast<unsigned char *>(p->d_rk) + half;
     cudaStream_t s = (cudaStream_t)stream;
     const int prec = ds.prec == EF_PREC_F32 ? 0 : 1;
-    const SplitUse use(p, ncells, s);
+    const WorkUse use(p, ncells, s, true);
     for (int k = 0; k < nsteps; ++k) {
         double *dk = diag ? diag + (int64_t)k * ncells * ef::kDiag : nullptr;
         // F1 = F + dt Q[F]
