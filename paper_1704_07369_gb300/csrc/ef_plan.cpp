@@ -256,9 +256,11 @@ struct ClassPlan {
     Shape cur{};                        // the shape of the fields above
     std::vector<Shape> shapes;          // uniform: the shapes a call may choose from by its cell count
     int pin_split = 0;                  // > 0: parts per cell pinned with the shape
-    int64_t pick_n = -1;                // the last choice: cell count, shape, parts
-    size_t pick_i = 0;
-    int pick_s = 1;
+    struct Pick {                       // the last choice without [0] and with [1] parts
+        int64_t n = -1;
+        size_t shape = 0;
+        int parts = 1;
+    } pick[2];
     // kWorkSlots workspaces of each kind that the class needs, *_bytes one of them
     void *d_part = nullptr;             // gains of the parts of split launches
     size_t part_bytes = 0;
@@ -541,32 +543,33 @@ double launch_cycles(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64
     return t;
 }
 
-// The shape and parts of a call on n cells of a uniform plan.  The plan's first shape (the smallest
-// cluster that fits) is kept unless another one, or a split, is estimated at least a tenth faster.
-void pick_shape(const Desc &ds, ClassPlan &cp, int64_t n, int sms)
+// The shape and parts of a call on n cells of a uniform plan, split = false: of one that may not be split (its
+// own choice: the best shape for parts may be a slow one for whole cells).  The plan's first shape (the
+// smallest cluster that fits) is kept unless another one, or a split, is estimated at least a tenth faster.
+const ClassPlan::Pick &pick_shape(const Desc &ds, ClassPlan &cp, int64_t n, bool split, int sms)
 {
-    if (cp.pick_n == n) return;
-    cp.pick_n = n;
-    cp.pick_i = 0;
-    cp.pick_s = 1;
+    ClassPlan::Pick &pk = cp.pick[split ? 1 : 0];
+    if (pk.n == n) return pk;
+    pk = ClassPlan::Pick{n, 0, 1};
     if (cp.pin_split > 0) {
-        cp.pick_s = std::min(cp.pin_split, max_split(ds, cp, cp.shapes[0], n));
-        return;
+        if (split) pk.parts = std::min(cp.pin_split, max_split(ds, cp, cp.shapes[0], n));
+        return pk;
     }
     double tb = 0.9 * launch_cycles(ds, cp, cp.shapes[0], n, 1, sms);
     const int u = units_of(cp);
     for (size_t i = 0; i < cp.shapes.size(); ++i) {
-        const int sm = max_split(ds, cp, cp.shapes[i], n);
+        const int sm = split ? max_split(ds, cp, cp.shapes[i], n) : 1;
         for (int k = 1; k <= sm; ++k) {
             if (k > 1 && (u + k - 1) / k == (u + k - 2) / (k - 1)) continue;      // no shorter longest part
             const double t = launch_cycles(ds, cp, cp.shapes[i], n, k, sms);
             if (t < tb) {
                 tb = t;
-                cp.pick_i = i;
-                cp.pick_s = k;
+                pk.shape = i;
+                pk.parts = k;
             }
         }
     }
+    return pk;
 }
 
 void apply_shape(ClassPlan &cp, const Shape &sh)
@@ -1132,9 +1135,9 @@ const Shape &call_shape(ef_plan_s *p, ClassPlan &cp, int64_t n, bool split, int 
         if (split) S = cp.split;
         return cp.cur;
     }
-    pick_shape(p->desc, cp, n, p->sms);
-    if (split) S = cp.pick_s;
-    return cp.shapes[cp.pick_i];
+    const ClassPlan::Pick &pk = pick_shape(p->desc, cp, n, split, p->sms);
+    S = pk.parts;
+    return cp.shapes[pk.shape];
 }
 
 // The workspace of one operation: slot >= 0, or -1 where its launches need none, or a capture finds none

@@ -161,3 +161,40 @@ def test_rk3_calls_wait_for_each_other(lib, prec):
         logs.append(p._log())
     assert logs[0][-1].kind == 2 and logs[1][0].kind == 3 and logs[1][0].event == logs[0][-1].event
     p.close()
+
+
+def call_info(p, n, split):
+    out = (ctypes.c_int64 * 8)()
+    assert p.lib.ef_plan_call_info(p.h, 0, ctypes.c_int64(n), split, out) == ef.EF_OK
+    return dict(zip(("parts", "cluster", "threads", "variant", "launches", "clusters"), out))
+
+
+@pytest.mark.parametrize("d,N,kernel,R,prec", SPECTRUM + [(3, 32, MAXWELL, 32, F32), (3, 48, HARD, 32, F32), (3, 32, MAXWELL, 32, F64)])
+@pytest.mark.parametrize("n", [1, 2, 7])
+def test_a_capture_without_a_workspace_launches_whole_cells(lib, d, N, kernel, R, prec, n):
+    """Four captures get workspaces; the fifth launches what ef_plan_call_info gives for a call that may not be
+    split."""
+    p = Plan(lib, d, N, kernel, R, prec)
+    split, whole = call_info(p, n, 1), call_info(p, n, 0)
+    assert whole["parts"] == 1 and whole["launches"] == 1
+    for g in range(5):
+        stream = 0x100 + 16 * g
+        lib.fake_begin_capture(ctypes.c_void_p(stream), ctypes.c_ulonglong(g + 1))
+        r = launches(p.collide(n, stream))[0]
+        lib.fake_end_capture(ctypes.c_void_p(stream))
+        want = split if g < 4 else whole
+        assert (r.nsplit, r.cluster, r.threads, r.occ) == (want["parts"], want["cluster"], want["threads"], want["variant"])
+    for g in range(5):
+        lib.fake_destroy_graph(ctypes.c_ulonglong(g + 1))
+    p.close()
+
+
+@pytest.mark.parametrize("d,N,kernel,R,prec,n", [(3, 16, HARD, 16, F64, 2), (3, 16, HARD, 16, F64, 4), (2, 64, MAXWELL, 16, F64, 2)])
+def test_whole_cells_do_not_take_the_shape_chosen_for_parts(lib, d, N, kernel, R, prec, n):
+    """Here parts run best one line transform a team on many small CTAs; a whole cell, whose every pass ends in
+    a cluster barrier, on fewer."""
+    p = Plan(lib, d, N, kernel, R, prec)
+    split, whole = call_info(p, n, 1), call_info(p, n, 0)
+    assert split["parts"] > 1 and whole["parts"] == 1
+    assert whole["cluster"] < split["cluster"]
+    p.close()
