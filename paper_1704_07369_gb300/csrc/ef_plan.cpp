@@ -696,7 +696,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
                 apply_shape(cp, sh);
                 cp.prefetch = pf;
                 // the key's bucket holds other cell counts: at most the parts this count allows
-                cp.split = may_split ? std::max(1, std::min(parts, max_split(ds, cp, sh, ncells_tune))) : 1;
+                cp.split = may_split ? std::max(1, std::min(parts, max_split(ds, cp, sh, cp.ncells))) : 1;
                 return EF_OK;
             }
     }
@@ -714,7 +714,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
     int64_t fh_need = 0;
     // clusters a timed launch may have: a split one has an item for every part
     auto clusters_of = [&](const Shape &sh) {
-        return std::min<int64_t>(ncells_tune * (may_split ? max_split(ds, cp, sh, ncells_tune) : 1), sh.max_clusters);
+        return std::min<int64_t>(ncells_tune * (may_split ? max_split(ds, cp, sh, cp.ncells) : 1), sh.max_clusters);
     };
     for (const Shape &sh : shapes) fh_need = std::max<int64_t>(fh_need, clusters_of(sh));
     if (e == cudaSuccess) e = cudaMalloc(&fhws, (size_t)fh_need * ef::collide_fh_bytes(ds.prec, d, cp.N));
@@ -724,7 +724,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
     int64_t part_cells = 0;
     if (may_split)
         for (const Shape &sh : shapes) {
-            const int S = max_split(ds, cp, sh, ncells_tune);
+            const int S = max_split(ds, cp, sh, cp.ncells);
             if (S > 1) part_cells = std::max<int64_t>(part_cells, ncells_tune * (S + 1));
         }
     if (e == cudaSuccess && part_cells) e = cudaMalloc(&parts_ws, (size_t)part_cells * cell * el);
@@ -794,7 +794,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
             e = cudaMalloc(&sgws, (size_t)grid * sh.cluster * 2 * rows * cp.N * el);
             if (e != cudaSuccess) break;
         }
-        const int smax = may_split ? max_split(ds, cp, sh, ncells_tune) : 1;
+        const int smax = may_split ? max_split(ds, cp, sh, cp.ncells) : 1;      // of the class, also where fewer cells are timed
         for (int v = 0; v < (smax > 1 ? 4 : 2) && e == cudaSuccess; ++v) {
             const int pfv = v & 1, split = v >= 2 ? smax : 1;
             double tmin = 1e30;

@@ -70,11 +70,12 @@ cudaError_t launch(int64_t kind, int N, const ef::CollideArgs &a, int grid, int 
     return cudaSuccess;
 }
 
-// resident clusters as a GB300 would have them: 152 SMs, 228 KB each, 64K registers (128 a thread; the
-// register kernels one CTA per SM), at most 32 CTAs
-int resident(size_t smem, int cluster, int tpb, bool one_per_sm)
+// resident clusters as a GB300 would have them: 152 SMs, 228 KB each, 64K registers (128 a thread, 32 for the
+// smallest cells; the register kernels one CTA per SM), at most 32 CTAs
+int resident(int N, size_t smem, int cluster, int tpb, bool one_per_sm)
 {
-    int per_sm = one_per_sm ? 1 : std::min<int>(32, std::min<int>((int)(228 * 1024 / (smem + 1024)), 65536 / (128 * tpb)));
+    const int regs = N <= 8 ? 32 : 128;
+    int per_sm = one_per_sm ? 1 : std::min<int>(32, std::min<int>((int)(228 * 1024 / (smem + 1024)), 65536 / (regs * tpb)));
     return per_sm * 152 / cluster;
 }
 
@@ -256,9 +257,9 @@ namespace ef {
     {                                                                                                                     \
         return occ >= 3 ? rg_smem(N, planes) : smem_bytes(EL, D, N, planes, sg, paired);                                  \
     }                                                                                                                     \
-    cudaError_t collide_setup_##SUF(int, size_t smem, int cluster, int tpb, int occ, int *mc)                             \
+    cudaError_t collide_setup_##SUF(int N, size_t smem, int cluster, int tpb, int occ, int *mc)                           \
     {                                                                                                                     \
-        *mc = resident(smem, cluster, tpb, occ >= 3);                                                                     \
+        *mc = resident(N, smem, cluster, tpb, occ >= 3);                                                                    \
         return cudaSuccess;                                                                                               \
     }                                                                                                                     \
     cudaError_t collide_launch_##SUF(int N, const CollideArgs &a, int grid, int tpb, size_t, int occ, cudaStream_t s)     \
@@ -272,9 +273,9 @@ EF_FAKE_VARIANT(f64_3d, 8, 3)
 
 int rg_rows_per_thread(int v) { return v == 2 ? 2 : 1; }
 int rg_team(int) { return 1; }
-cudaError_t rg_split_setup_f32(int, int, size_t smem, int cluster, int tpb, int *mc)
+cudaError_t rg_split_setup_f32(int N, int, size_t smem, int cluster, int tpb, int *mc)
 {
-    *mc = resident(smem, cluster, tpb, true);
+    *mc = resident(N, smem, cluster, tpb, true);
     return cudaSuccess;
 }
 cudaError_t rg_split_launch_f32(int N, int v, const CollideArgs &a, int grid, int tpb, size_t, cudaStream_t s)

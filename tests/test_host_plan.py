@@ -198,3 +198,17 @@ def test_whole_cells_do_not_take_the_shape_chosen_for_parts(lib, d, N, kernel, R
     assert split["parts"] > 1 and whole["parts"] == 1
     assert whole["cluster"] < split["cluster"]
     p.close()
+
+
+@pytest.mark.parametrize("n,split", [(400, True), (2400, True), (3000, False), (6000, False), (200000, False)])
+def test_ragged_plans_split_only_what_is_resident_at_once(lib, n, split):
+    """Every part of a split launch has a cluster of its own, whatever smaller count the tuner timed: small cells
+    are resident by the thousand, and parts of more would be rounds of repeated work and workspaces that grow
+    with the batch."""
+    p = Plan(lib, 2, None, MAXWELL, 16, F32, cells=[8] * n)
+    used = lib.fake_used()
+    r = launches(p.collide(n))[0]
+    assert (r.nsplit > 1) == split
+    assert r.clusters >= n * r.nsplit or r.nsplit == 1
+    assert used <= (64 << 20) + 64 * n
+    p.close()
