@@ -261,7 +261,8 @@ struct ClassPlan {
         size_t shape = 0;
         int parts = 1;
     } pick[2];
-    // kWorkSlots workspaces of each kind that the class needs, *_bytes one of them
+    bool no_parts = false;              // no memory for the parts of split launches: calls are not split
+    // ef_plan_s::nslots workspaces of each kind that the class needs, *_bytes one of them
     void *d_part = nullptr;             // gains of the parts of split launches
     size_t part_bytes = 0;
     void *d_fin = nullptr;              // arrivals and diagnostics of the finishing launches
@@ -341,6 +342,7 @@ struct ef_plan_s {
     cudaEvent_t work_done = nullptr;
     bool work_used = false;
     std::shared_ptr<WorkSlots> slots;
+    int nslots = kWorkSlots;            // 1 where there was no memory for the captures' workspaces
     // SSP-RK3 stage buffers: two batch-sized arrays, grown on demand
     void *d_rk = nullptr;
     size_t rk_bytes = 0;
@@ -494,6 +496,9 @@ std::vector<Shape> candidate_shapes(const Desc &ds, int N, std::string &why)
     return out;
 }
 
+// Parts per cell of a batched plan's launches.
+int call_split(const ClassPlan &cp) { return cp.no_parts ? 1 : cp.split; }
+
 // Parts per cell a launch of n cells may use: all its items resident at once, at most one part per unit
 // (a pair of transforms, or the loss), and only the kernels built for it.
 int units_of(const ClassPlan &cp) { return (cp.nops_paired > 0 ? cp.nops_paired : 1); }
@@ -501,7 +506,7 @@ int units_of(const ClassPlan &cp) { return (cp.nops_paired > 0 ? cp.nops_paired 
 int max_split(const Desc &ds, const ClassPlan &cp, const Shape &sh, int64_t n)
 {
     if (ds.prec == EF_PREC_F32 && ds.d == 3 && sh.occ != 1 && sh.occ != 3 && sh.occ != 4) return 1;
-    if (n <= 0 || n >= sh.max_clusters) return 1;
+    if (cp.no_parts || n <= 0 || n >= sh.max_clusters) return 1;
     return (int)std::max<int64_t>(1, std::min<int64_t>(units_of(cp), sh.max_clusters / n));
 }
 
@@ -659,6 +664,7 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
         return fail(EF_ERR_UNSUPPORTED, "no launch shape fits N=" + std::to_string(cp.N) + " on this device " + why);
     apply_shape(cp, shapes[0]);
     cp.prefetch = 0;
+    cp.shapes.clear();
     // a uniform plan's call chooses by its cell count: the first shape, and for the register kernels the
     // instantiations that can be split
     for (const Shape &sh : shapes)
@@ -847,6 +853,10 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
     if (st) cudaStreamDestroy(st);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
+    if (e == cudaErrorMemoryAllocation && may_split) {
+        cudaGetLastError();                        // split launches need more: time whole cells only
+        return choose_shape(ds, cp, ncells_tune, false, sms);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "autotune");
     apply_shape(cp, best_sh);
     cp.prefetch = best_pf;
@@ -989,7 +999,7 @@ ef_status build_class(const Desc &ds, ClassPlan &cp, bool may_split, int sms)
 
 // Workspaces of one class for every cluster that can be resident at once (max_clusters, fixed by the
 // launch shapes): forward spectra, S/G accumulators of the global-accumulator shapes, and the parts of
-// split launches.  Called once at plan creation, so that no operation allocates.
+// split launches (unless cp.no_parts).  Called at plan creation, so that no operation allocates.
 ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
 {
     const Desc &ds = p->desc;
@@ -1005,14 +1015,14 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
         if (!p->batched && max_split(ds, cp, sh, 1) > 1) fin_cells = std::max<int64_t>(fin_cells, sh.max_clusters);
         if (!p->batched && max_split(ds, cp, sh, 1) > 1) part_cells = std::max<int64_t>(part_cells, sh.max_clusters + (sh.max_clusters + 1) / 2);
     }
-    if (p->batched && cp.split > 1) {
-        part_cells = cp.ncells * (cp.split + 1);
+    if (p->batched && call_split(cp) > 1) {
+        part_cells = cp.ncells * (call_split(cp) + 1);
         fin_cells = cp.ncells;
     }
     auto alloc = [&](void **q, size_t &bytes, size_t need) {
         bytes = (need + 255) / 256 * 256;
         if (!bytes) return cudaSuccess;
-        const cudaError_t e = cudaMalloc(q, kWorkSlots * bytes);
+        const cudaError_t e = cudaMalloc(q, p->nslots * bytes);
         if (e != cudaSuccess) *q = nullptr;
         return e;
     };
@@ -1024,11 +1034,20 @@ ef_status alloc_workspaces(ef_plan_s *p, ClassPlan &cp)
         e = alloc(&cp.d_part, cp.part_bytes, (size_t)part_cells * cell * el);
         cp.fin_off = fin_offset(fin_cells);
         if (e == cudaSuccess) e = alloc(&cp.d_fin, cp.fin_bytes, cp.fin_off + fin_diag_bytes(fin_cells, p->sms));
-        if (e == cudaSuccess) e = cudaMemset(cp.d_fin, 0, kWorkSlots * cp.fin_bytes);
+        if (e == cudaSuccess) e = cudaMemset(cp.d_fin, 0, p->nslots * cp.fin_bytes);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();      // whatever stream the first call is on
         if (e != cudaSuccess) return cuda_fail(e, "part workspace");
     }
     return EF_OK;
+}
+
+void workspaces_free(ClassPlan &cp)
+{
+    for (void **q : {&cp.d_fh, &cp.d_sg, &cp.d_part, &cp.d_fin}) {
+        cudaFree(*q);
+        *q = nullptr;
+    }
+    cp.fh_bytes = cp.sg_bytes = cp.part_bytes = cp.fin_bytes = 0;
 }
 
 // The launch fits the workspaces made at plan creation (always true, since the grid never exceeds
@@ -1052,10 +1071,7 @@ void destroy_plan(ef_plan_s *p)
         cudaFree(cp.d_ops_paired);
         cudaFree(cp.d_cell_off);
         cudaFree(cp.d_cell_id);
-        cudaFree(cp.d_sg);
-        cudaFree(cp.d_fh);
-        cudaFree(cp.d_part);
-        cudaFree(cp.d_fin);
+        workspaces_free(cp);
     }
     if (p->work_done) cudaEventDestroy(p->work_done);
     cudaFree(p->d_all_off);
@@ -1132,7 +1148,7 @@ const Shape &call_shape(ef_plan_s *p, ClassPlan &cp, int64_t n, bool split, int 
 {
     S = 1;
     if (p->batched) {
-        if (split) S = cp.split;
+        if (split) S = call_split(cp);
         return cp.cur;
     }
     const ClassPlan::Pick &pk = pick_shape(p->desc, cp, n, split, p->sms);
@@ -1176,12 +1192,12 @@ struct WorkUse {
         if (!needs || cap != cudaStreamCaptureStatusActive) return true;
         if (capture_info(s, &cap, &capture, &graph) != cudaSuccess) return false;
         WorkSlots &ws = *p->slots;
-        for (int i = 1; i < kWorkSlots; ++i)
+        for (int i = 1; i < p->nslots; ++i)
             if (ws.taken[i].load() && ws.capture[i] == capture && ws.stream[i] == s) {
                 slot = i;
                 return true;
             }
-        for (int i = 1; i < kWorkSlots; ++i) {
+        for (int i = 1; i < p->nslots; ++i) {
             int free_ = 0;
             if (!ws.taken[i].compare_exchange_strong(free_, 1)) continue;
             WorkLease *l = new WorkLease{p->slots, i};
@@ -1317,8 +1333,20 @@ ef_status finish_plan(ef_plan_s *p)
     for (ClassPlan &cp : p->classes) {
         ef_status st = build_class(p->desc, cp, p->may_split, p->sms);
         if (st != EF_OK) return st;
-        st = alloc_workspaces(p, cp);
-        if (st != EF_OK) return st;
+    }
+    // Only what whole cells need has to fit: without room for the captures' workspaces the plan's captures
+    // share the calls', without room for parts its calls are not split.
+    for (int need = 0;; ++need) {
+        ef_status st = EF_OK;
+        for (ClassPlan &cp : p->classes)
+            if (st == EF_OK) st = alloc_workspaces(p, cp);
+        if (st == EF_OK) break;
+        for (ClassPlan &cp : p->classes) workspaces_free(cp);
+        if (st != EF_ERR_OOM || need == 2) return st;
+        cudaGetLastError();
+        p->nslots = 1;
+        if (need == 1)
+            for (ClassPlan &cp : p->classes) cp.no_parts = true;
     }
     if (p->classes.size() > 1) {
         e = cudaMalloc((void **)&p->d_counters, p->classes.size() * sizeof(unsigned long long));

@@ -27,6 +27,7 @@ std::vector<FakeRec> g_log;
 std::map<void *, size_t> g_mem;
 size_t g_used = 0, g_peak = 0, g_limit = (size_t)1 << 40;
 double g_clock = 0.0;
+cudaError_t g_error = cudaSuccess;
 std::map<cudaStream_t, unsigned long long> g_capture;            // capturing streams
 std::map<unsigned long long, std::vector<cudaUserObject_t>> g_graphs;
 intptr_t g_next = 0x1000;
@@ -99,6 +100,12 @@ int64_t fake_log(FakeRec *out, int64_t n)
 void fake_clear(void) { g_log.clear(); }
 void fake_limit(size_t bytes) { g_limit = bytes; }
 size_t fake_used(void) { return g_used; }
+size_t fake_peak(void)
+{
+    const size_t p = g_peak;
+    g_peak = g_used;
+    return p;
+}
 void fake_begin_capture(void *s, unsigned long long id)
 {
     g_capture[(cudaStream_t)s] = id;
@@ -117,10 +124,11 @@ void fake_destroy_graph(unsigned long long id)
 
 cudaError_t cudaMalloc(void **p, size_t n)
 {
-    if (g_used + n > g_limit) return cudaErrorMemoryAllocation;
+    if (g_used + n > g_limit) return g_error = cudaErrorMemoryAllocation;
     *p = std::aligned_alloc(256, (n + 255) / 256 * 256 + 256);
     g_mem[*p] = n;
     g_used += n;
+    g_peak = std::max(g_peak, g_used);
     return cudaSuccess;
 }
 cudaError_t cudaFree(void *p)
@@ -162,7 +170,13 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int)
     p->multiProcessorCount = 152;
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetLastError(void)
+{
+    const cudaError_t e = g_error;
+    g_error = cudaSuccess;
+    return e;
+}
+cudaError_t cudaPeekAtLastError(void) { return g_error; }
 const char *cudaGetErrorString(cudaError_t) { return "fake error"; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned)
 {

@@ -30,6 +30,7 @@ def lib(tmp_path_factory):
     lib = ctypes.CDLL(out)
     lib.fake_log.restype = ctypes.c_int64
     lib.fake_used.restype = ctypes.c_size_t
+    lib.fake_peak.restype = ctypes.c_size_t
     lib.ef_last_error.restype = ctypes.c_char_p
     return lib
 
@@ -212,3 +213,44 @@ def test_ragged_plans_split_only_what_is_resident_at_once(lib, n, split):
     assert r.clusters >= n * r.nsplit or r.nsplit == 1
     assert used <= (64 << 20) + 64 * n
     p.close()
+
+
+@pytest.mark.parametrize("d,N,kernel,R,prec,cells", [(3, 32, MAXWELL, 32, F32, None), (3, 32, HARD, 32, F64, None), (2, 64, MAXWELL, 16, F64, None),
+                                                     (3, 64, HARD, 16, F64, None), (3, None, HARD, 32, F32, [32] * 20 + [48] * 3)])
+def test_a_plan_without_room_for_parts_and_captures_still_works(lib, d, N, kernel, R, prec, cells):
+    """The workspaces of split launches and of captures are dropped before a plan is refused: down to what whole
+    cells need, every limit of device memory below the full plan's is enough, and nothing is left behind."""
+    n = 1 if cells is None else len(cells)
+    base = lib.fake_used()
+    lib.fake_peak()
+    p = Plan(lib, d, N, kernel, R, prec, cells)
+    full = lib.fake_peak() - base
+    assert any(r.nsplit > 1 for r in launches(p.collide(n)))
+    p.close()
+    assert lib.fake_used() == base
+    kinds = set()
+    frac = 1.0
+    try:
+        while True:
+            frac *= 0.75
+            lib.fake_limit(ctypes.c_size_t(base + int(full * frac)))
+            h = ctypes.c_void_p()
+            try:
+                p = Plan(lib, d, N, kernel, R, prec, cells)
+            except AssertionError:
+                break
+            assert lib.cudaPeekAtLastError() == 0
+            log = p.collide(n)
+            kinds.add(any(r.nsplit > 1 for r in launches(log)))
+            lib.fake_begin_capture(ctypes.c_void_p(0x100), ctypes.c_ulonglong(1))
+            captured = p.collide(n, 0x100)
+            lib.fake_end_capture(ctypes.c_void_p(0x100))
+            assert len(launches(captured)) == len(launches(log))
+            lib.fake_destroy_graph(ctypes.c_ulonglong(1))
+            p.close()
+            assert lib.fake_used() == base
+    finally:
+        lib.fake_limit(ctypes.c_size_t(1 << 40))
+    assert lib.fake_used() == base
+    assert kinds == {True, False}
+    assert frac <= 0.35
