@@ -800,12 +800,20 @@ ef_status choose_shape(const Desc &ds, ClassPlan &cp, int64_t ncells_tune, bool 
             e = cudaMalloc(&sgws, (size_t)grid * sh.cluster * 2 * rows * cp.N * el);
             if (e != cudaSuccess) break;
         }
+        // whole cells with and without the prefetch (the FP64 kernel has none), then parts with the better one
         const int smax = may_split ? max_split(ds, cp, sh, cp.ncells) : 1;      // of the class, also where fewer cells are timed
-        for (int v = 0; v < (smax > 1 ? 4 : 2) && e == cudaSuccess; ++v) {
-            const int pfv = v & 1, split = v >= 2 ? smax : 1;
+        const int npf = ds.prec == EF_PREC_F32 ? 2 : 1;
+        int pf_best = 0;
+        double whole = 1e30;
+        for (int v = 0; v < npf + (smax > 1 ? 1 : 0) && e == cudaSuccess; ++v) {
+            const int pfv = v < npf ? v : pf_best, split = v < npf ? 1 : smax;
             double tmin = 1e30;
             e = time_one(sh, pfv, split, n1, tmin);
             if (e != cudaSuccess) break;
+            if (v < npf && tmin < whole) {
+                whole = tmin;
+                pf_best = pfv;
+            }
             sweep.push_back(Timed{tmin, i, pfv, split});
             // EF_AUTOTUNE_LOG names a file that receives every timed candidate (tuning records)
             if (const char *lp = std::getenv("EF_AUTOTUNE_LOG")) {

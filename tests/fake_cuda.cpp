@@ -18,7 +18,7 @@ struct FakeRec {
     int64_t kind;        // 0 collide, 1 finish, 2 event record, 3 event wait, 4 other kernel
     int64_t stream, event;
     int64_t N, ncells, cells_off, nsplit, cluster, threads, occ, sg_global, clusters;
-    int64_t fh, sg, part, fin;
+    int64_t fh, sg, part, fin, paired, prefetch;
 };
 
 namespace {
@@ -66,6 +66,8 @@ cudaError_t launch(int64_t kind, int N, const ef::CollideArgs &a, int grid, int 
     r.sg = (int64_t)(intptr_t)a.sg_ws;
     r.part = (int64_t)(intptr_t)a.part;
     r.fin = (int64_t)(intptr_t)a.fin;
+    r.paired = a.paired;
+    r.prefetch = a.prefetch;
     g_log.push_back(r);
     g_clock += kind == 0 ? 1.0 / a.nsplit + 0.001 * a.cluster : 0.01;      // split launches tune as the faster ones
     return cudaSuccess;

@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(ROOT, "paper_1704_07369_gb300", "csrc")
 
 FIELDS = ("kind", "stream", "event", "N", "ncells", "cells_off", "nsplit", "cluster", "threads", "occ", "sg_global",
-          "clusters", "fh", "sg", "part", "fin")
+          "clusters", "fh", "sg", "part", "fin", "paired", "prefetch")
 
 
 class _Rec(ctypes.Structure):
@@ -254,3 +254,30 @@ def test_a_plan_without_room_for_parts_and_captures_still_works(lib, d, N, kerne
     assert lib.fake_used() == base
     assert kinds == {True, False}
     assert frac <= 0.35
+
+
+@pytest.mark.parametrize("d,N,R,prec,kernel", [(3, 24, 16, F64, HARD), (2, 32, 16, F64, MAXWELL), (3, 24, 16, F32, HARD), (2, 16, 16, F32, MAXWELL)])
+def test_the_tuner_times_nothing_twice(lib, d, N, R, prec, kernel):
+    """Four launches of each candidate: whole cells, in FP32 with and without the prefetch, and parts with the
+    better of the two (the FP64 kernel has no prefetch)."""
+    h = ctypes.c_void_p()
+    cells = [N] * 20
+    lib.fake_clear()
+    assert lib.ef_plan_create_batched(d, ctypes.c_int64(20), (ctypes.c_int * 20)(*cells), ctypes.c_double(8.0), kernel, R, prec,
+                                      ctypes.byref(h)) == ef.EF_OK
+    buf = (_Rec * 8192)()
+    n = lib.fake_log(buf, ctypes.c_int64(8192))
+    lib.fake_clear()
+    assert n <= 8192
+    timed = {}
+    for r in launches(buf[:n]):
+        shape = (r.cluster, r.threads, r.occ, r.sg_global, r.paired)
+        timed.setdefault(shape, {}).setdefault((r.nsplit, r.prefetch), 0)
+        timed[shape][(r.nsplit, r.prefetch)] += 1
+    assert timed
+    for shape, forms in timed.items():
+        assert set(forms.values()) == {4}
+        whole = [f for f in forms if f[0] == 1]
+        assert len(whole) == (1 if prec == F64 else 2)
+        assert len(forms) - len(whole) <= 1
+    lib.ef_plan_destroy(h)
