@@ -28,12 +28,13 @@ namespace ef {
 
 namespace cg = cooperative_groups;
 
-// Threads per CTA the kernel is compiled for.  Registers are shared per SM sub-partition: 8 warps
-// allow 255 per thread, 10 warps (3 on some sub-partition) 168.  The output pass (Q or F + dt Q
-// with the FP64 diagnostics) holds three rows of N values; FP32 N >= 40 and FP64 keep 8 warps so
-// that it does not spill (the plan-time autotuner picks smaller CTAs in any case).
-template <typename T, int N>
-__host__ __device__ constexpr int max_threads() { return (sizeof(T) == 8 || N >= 40) ? 256 : 320; }
+// Threads per CTA the kernel is compiled for (FP32; FP64 has a kernel of its own, ef_collide_q.cuh).
+// Registers are shared per SM sub-partition: 8 warps allow 255 per thread, 10 warps (3 on some
+// sub-partition) 168.  The output pass (Q or F + dt Q with the FP64 diagnostics) holds three rows of N
+// values; N >= 40 keeps 8 warps so that it does not spill (the plan-time autotuner picks smaller CTAs
+// in any case).
+template <int N>
+__host__ __device__ constexpr int max_threads() { return N >= 40 ? 256 : 320; }
 
 // Second instantiation for two co-resident CTAs per SM (of different cells, whose barrier phases
 // then overlap): at most 6 warps per CTA, so 12 per SM and 168 registers per thread.  Built for
@@ -275,13 +276,6 @@ __device__ __forceinline__ void load_row(const T *src, T (&x)[N])
             const float4 v = s4[i];
             x[4 * i] = v.x; x[4 * i + 1] = v.y; x[4 * i + 2] = v.z; x[4 * i + 3] = v.w;
         }
-    } else if constexpr (sizeof(T) == 8 && N % 2 == 0) {
-        const double2 *s2 = reinterpret_cast<const double2 *>(src);
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            const double2 v = s2[i];
-            x[2 * i] = v.x; x[2 * i + 1] = v.y;
-        }
     } else {
 #pragma unroll
         for (int n = 0; n < N; ++n) x[n] = src[n];
@@ -295,10 +289,6 @@ __device__ __forceinline__ void store_row(T *dst, const T (&x)[N])
         float4 *d4 = reinterpret_cast<float4 *>(dst);
 #pragma unroll
         for (int i = 0; i < N / 4; ++i) d4[i] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
-    } else if constexpr (sizeof(T) == 8 && N % 2 == 0) {
-        double2 *d2 = reinterpret_cast<double2 *>(dst);
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) d2[i] = make_double2(x[2 * i], x[2 * i + 1]);
     } else {
 #pragma unroll
         for (int n = 0; n < N; ++n) dst[n] = x[n];
@@ -532,8 +522,9 @@ __device__ __forceinline__ void diag_reduce_f64(const CollideArgs &a, Diag &dg, 
 }
 
 template <typename T, int D, int N, int OCC = 1>
-__global__ void __launch_bounds__(OCC == 1 ? max_threads<T, N>() : kOcc2Threads, OCC) collide_kernel(const CollideArgs a)
+__global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OCC) collide_kernel(const CollideArgs a)
 {
+    static_assert(sizeof(T) == 4, "FP32; FP64: collide_kernel_q");
     constexpr int H = N / 2 + 1;
     constexpr int N1 = (D == 3) ? N : 1;
     constexpr int NP = N1 * H;         // spectral columns of one axis-0 plane = pencils

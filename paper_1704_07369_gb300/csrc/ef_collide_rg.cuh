@@ -326,6 +326,7 @@ template <int D, int N, int RPT, int LB, bool GS, bool ASYNC, bool SPLIT = false
 __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
 {
     static_assert(D == 3, "3D only");
+    static_assert(!(GS && SPLIT), "split launches keep G in registers");
     using T = float;
     constexpr int NPP = rg_plane_stride<N>();
     constexpr int NH = N / 2;              // stored k_x values per row
@@ -465,15 +466,11 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
         DiagF dg;
         T g[GS ? 1 : RPT][N];              // G in registers: this thread's rows tid + j nt
 
-        if (S > 1) {
-            if constexpr (GS) {
-                for (int i = tid; i < rows * N; i += nt) Gs[i] = T(0);       // read after later barriers
-            } else {
+        if constexpr (SPLIT) {
 #pragma unroll
-                for (int j = 0; j < RPT; ++j)
+            for (int j = 0; j < RPT; ++j)
 #pragma unroll
-                    for (int n = 0; n < N; ++n) g[j][n] = T(0);
-            }
+                for (int n = 0; n < N; ++n) g[j][n] = T(0);
         }
 
         for (int o = o0; o < o1; ++o) {
@@ -694,21 +691,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             continue;
         }
 
-        if (S > 1) {                       // this part's gain (zeros from a part with only the loss)
+        if constexpr (SPLIT) {             // this part's gain (zeros from a part with only the loss)
             T *pg = reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL + (int64_t)rank * rows * N;
-            if constexpr (GS) {
-                __syncthreads();
-                for (int r = tid; r < rows; r += nt) {
-                    T gv[N];
 #pragma unroll
-                    for (int n = 0; n < N; ++n) gv[n] = Gs[n * rows + r];
-                    store_row<T, N>(pg + (int64_t)r * N, gv);
-                }
-                __syncthreads();
-            } else {
-#pragma unroll
-                for (int j = 0; j < RPT; ++j) store_row<T, N>(pg + (int64_t)(tid + j * nt) * N, g[j]);
-            }
+            for (int j = 0; j < RPT; ++j) store_row<T, N>(pg + (int64_t)(tid + j * nt) * N, g[j]);
             continue;
         }
 

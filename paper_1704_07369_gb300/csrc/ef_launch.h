@@ -74,10 +74,10 @@ struct PlanView {
     int device;
 };
 bool plan_view(const struct ef_plan_s *p, PlanView *out);
-// uniform plan on the doubled grid 2N with multipliers restricted to the N grid's Galerkin modes
 // ef_plan_create_batched; may_split = false for plans whose steps run side by side on several streams
 ef_status ef_plan_create_batched_opt(int d, int64_t ncells, const int *N_host, double L, ef_kernel kernel, int R, ef_precision prec,
                               bool may_split, struct ef_plan_s **out);
+// uniform plan on the doubled grid 2N with multipliers restricted to the N grid's Galerkin modes
 ef_status plan_create_padded(const ef_plan_desc *desc, struct ef_plan_s **out);
 // forward pass of n on the input that the last forward pass of `first` on this stream packed (ef_mlp.cu)
 ef_status mlp_forward_same_input(ef_mlp_t n, ef_mlp_t first, float *Y, int ldy, int64_t B, cudaStream_t s);
@@ -126,10 +126,10 @@ EF_DECLARE_FEAT(f32)
 EF_DECLARE_FEAT(f64)
 #undef EF_DECLARE_FEAT
 
-// out = a x + b y over n values (ef_step.cu); prec 0 = FP32, 1 = FP64
 // free transport between the spatial cells of a uniform batch (ef_transport.cu), c = dt h / dx
 cudaError_t transport_launch(int prec, int d, int N, const void *Fin, void *Fout, int64_t ncells, double c,
                              cudaStream_t s);
+// out = a x + b y over n values (ef_step.cu); prec 0 = FP32, 1 = FP64
 cudaError_t axpby_launch(int prec, void *out, const void *x, const void *y, double a, double b, int64_t n,
                          cudaStream_t s);
 
