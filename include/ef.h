@@ -214,8 +214,9 @@ ef_status ef_mlp_destroy(ef_mlp_t mlp);
 ef_status ef_mlp_info(ef_mlp_t mlp, int64_t info[8]);
 
 /* The MLP's device status word, as ef_plan_status does for a plan: EF_OK, or EF_ERR_TIMEOUT when a
- * tensor-core GEMM gave up one of its bounded mbarrier waits (that GEMM's outputs are then NaN and
- * the work queued after it on the stream saw them).  sync = 1 synchronises the device and reads
+ * tensor-core GEMM gave up one of its bounded mbarrier waits (the outputs that the CTA had still to
+ * write are then NaN, those it had written before stand, and the work queued after it on the stream
+ * saw them).  sync = 1 synchronises the device and reads
  * the word; sync = 0 returns the value last read.  reset = 1 clears it. */
 ef_status ef_mlp_status(ef_mlp_t mlp, int sync, int reset);
 

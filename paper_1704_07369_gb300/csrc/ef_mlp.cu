@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
                     }
                 }
                 if (!g.Cb && !g.CbT) continue;
-                if (g.relu) {
+                if (g.relu && ok) {              // (fmaxf would turn a given-up tile's NaN into 0)
 #pragma unroll
                     for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f);
                 }
