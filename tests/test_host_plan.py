@@ -26,7 +26,7 @@ def lib(tmp_path_factory):
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I" + os.path.join(cuda, "include"),
                     "-I" + os.path.join(ROOT, "include"), "-I" + CSRC, os.path.join(HERE, "fake_cuda.cpp"),
-                    os.path.join(CSRC, "ef_plan.cpp"), "-o", out, "-lpthread"], check=True)
+                    os.path.join(CSRC, "ef_plan.cpp"), "-o", out, "-lpthread", "-Wl,-Bsymbolic"], check=True)      # its own runtime, whatever else is loaded
     lib = ctypes.CDLL(out)
     lib.fake_log.restype = ctypes.c_int64
     lib.fake_used.restype = ctypes.c_size_t
@@ -234,7 +234,6 @@ def test_a_plan_without_room_for_parts_and_captures_still_works(lib, d, N, kerne
         while True:
             frac *= 0.75
             lib.fake_limit(ctypes.c_size_t(base + int(full * frac)))
-            h = ctypes.c_void_p()
             try:
                 p = Plan(lib, d, N, kernel, R, prec, cells)
             except AssertionError:
