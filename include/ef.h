@@ -224,7 +224,8 @@ ef_status ef_mlp_status(ef_mlp_t mlp, int sync, int reset);
 ef_status ef_mlp_params(ef_mlp_t mlp, float *host, int set);
 
 /* Y[b][0..padded nout) = mlp(X[b][0..nin)) for b < batch; X row stride ldx >= nin, Y row stride ldy
- * >= padded nout and even.  batch a multiple of 64, <= max_batch. */
+ * >= padded nout and even, Y on an 8-byte boundary (EF_ERR_INVALID_ARG otherwise).  batch a multiple of
+ * 64, <= max_batch. */
 ef_status ef_mlp_forward(ef_mlp_t mlp, const float *X, int ldx, float *Y, int ldy, int64_t batch, ef_stream_t stream);
 
 /* Mean squared error against T (row stride ldt >= nout) over the nout outputs, weighted by

@@ -1085,7 +1085,8 @@ ef_status ef_mlp_forward(ef_mlp_t n, const float *X, int ldx, float *Y, int ldy,
 {
     if (!n || !X || !Y) return mlp_fail(EF_ERR_INVALID_ARG, "null mlp, X or Y");
     if (B < 0 || B % 64 || B > n->max_batch) return mlp_fail(EF_ERR_INVALID_ARG, "batch must be a multiple of 64 <= max_batch");
-    if (ldx < n->nin || ldy < n->noutp || ldy % 2) return mlp_fail(EF_ERR_INVALID_ARG, "ldx >= nin, ldy >= padded nout (even)");
+    if (ldx < n->nin || ldy < n->noutp || ldy % 2 || (uintptr_t)Y % 8)
+        return mlp_fail(EF_ERR_INVALID_ARG, "ldx >= nin, ldy >= padded nout (even), Y 8-byte aligned");
     if (B == 0) return EF_OK;
     cudaStream_t s = (cudaStream_t)stream;
     pack_input_kernel<false><<<dim3((unsigned)(B / TT), n->ninp / TT), 256, 0, s>>>(X, ldx, n->nin, n->ninp, B, n->Xb, nullptr);
