@@ -19,7 +19,8 @@ policies (a checker network sends the cells it doubts to the plain operator, Q r
 grid) and the audit policies (none; any audited miss sends the whole batch to the plain operator;
 more than 5% of audited cells missing does).  --no-surrogate skips it.  The "hbm_kernels" object then times the
 library's HBM-bound kernels (moments / entropy and free transport) on resident N = 32 batches
-against the measured HBM copy rate; --no-kernels skips it.
+against the measured HBM copy rate; --no-kernels skips it.  The line carries these legs' figures of
+merit; their full reports go to standard error.
 
 --impl reference times the FP64 CPU oracle (direct O(R N^6) sum of the paper's operator) on the
 host cores, on a bounded sample of the same workload.
@@ -429,8 +430,42 @@ def run_ours(args, world, rank, local):
         line["cpu_baseline"] = cpu_baseline()
     elif not args.no_cpu_baseline:
         line["cpu_baseline"] = None
-    print(json.dumps(line), flush=True)
+    short, full = printed_line(line)
+    if full:
+        print("extra legs in full: " + json.dumps(full), file=sys.stderr, flush=True)
+    print(json.dumps(short), flush=True)
     return 0
+
+
+def printed_line(line):
+    """(the line to print, what it leaves out).  The extra legs' reports (surrogate, hbm_kernels, precision) run
+    to tens of kilobytes, and a reader that keeps only the end of the output would lose the line they are in: in
+    the line each is cut down to its figures of merit, and all of it goes to standard error."""
+    short, full = dict(line), {}
+
+    def num(x):
+        return float("%.5g" % x) if isinstance(x, float) else x
+
+    def pick(d, keys):
+        return {k: num(d[k]) for k in keys if k in d}
+
+    for leg in ("surrogate", "hbm_kernels", "precision"):
+        rep = line.get(leg)
+        if not isinstance(rep, dict):
+            continue
+        full[leg] = rep
+        if "error" in rep:
+            short[leg] = {"error": str(rep["error"])[:200]}
+        elif leg == "surrogate":
+            short[leg] = {k: dict(pick(r, ("plain_ms",)),
+                                  speedup_vs_plain={p: num(v["speedup_vs_plain"]) for p, v in r["policies"].items()})
+                          for k, r in rep.get("kernels", {}).items()}
+        elif leg == "hbm_kernels":
+            short[leg] = {k: num(v["frac_of_measured_hbm"]) for k, v in rep.items() if isinstance(v, dict)}
+        else:
+            short[leg] = {k: pick(v, ("fp32_ms", "fp64_ms", "fp32_ms_per_step", "fp64_ms_per_step", "gpu_ms_per_eval",
+                                      "gpu_ms_per_step", "oracle_ms_per_step")) for k, v in rep.items() if isinstance(v, dict)}
+    return short, full
 
 
 # -------------------------------------------------------------- precision and small configs -
@@ -828,7 +863,8 @@ def surrogate_leg(args, device):
 
 
 COLLIDE_SOURCES = ("ef_collide_impl.cuh", "ef_collide_rg.cuh", "ef_collide_tm.cuh", "ef_fft.cuh", "ef_internal.h",
-                   "ef_collide_variant.inc", "ef_collide_f32_3d.cu", "ef_collide_rg_f32.cu", "ef_collide_tm_f32.cu",
+                   "ef_collide_variant.inc", "ef_collide_f32_3d.cu", "ef_collide_rg_f32.cu", "ef_collide_rg_async_f32.cu",
+                   "ef_collide_rg_split_f32.cu", "ef_collide_tm_f32.cu",
                    "ef_cluster_launch.h")
 
 
