@@ -306,6 +306,14 @@ __device__ __forceinline__ void flag_cluster(cg::cluster_group &cl, int C, int *
         for (int r = 0; r < C; ++r) *cl.map_shared_rank(flag, r) = 1;
 }
 
+// A split launch's flag of each cell, dt nu > 1 somewhere in it: cleared and set by the part that holds the
+// loss, read by the finishing kernel (ef_split.cu).  (Findings that met in the finishing kernel itself cost a
+// small step 2 us of 12 - 19, for barriers or the latency of an atomic.)
+__device__ __forceinline__ unsigned *fin_flags(const CollideArgs &a)
+{
+    return reinterpret_cast<unsigned *>(static_cast<unsigned char *>(a.fin) + a.fin_off / 2);
+}
+
 // Final output of one real row: Q = q, written as Q (collide) or F + dt Q (Euler), with the
 // non-finite status check and the diagnostic sums of the row.  Returns whether an updated value
 // of an Euler step is below zero.
@@ -599,6 +607,8 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OC
         if (S > 1) {
             pnu = reinterpret_cast<T *>(a.part) + (c * (S + 1) + S) * CELL;
             pg = reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL;
+            // cleared by one thread, set in the loss op by any: cluster barriers lie between
+            if (rank == 0 && tid == 0 && (a.paired ? o0 == 0 : o1 == a.nops)) fin_flags(a)[c] = 0;
         }
         const int64_t coff = a.cell_off ? a.cell_off[c] : c * CELL;
         const int64_t cglob = a.cell_id ? a.cell_id[c] : c;
@@ -755,6 +765,11 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OC
                         T nu0[N], nu1[N];
 #pragma unroll
                         for (int n = 0; n < N; ++n) { nu0[n] = z[n].x; nu1[n] = z[n].y; }
+                        bool big = false;
+#pragma unroll
+                        for (int n = 0; n < N; ++n)
+                            if (T(a.dt) * nu0[n] > T(1) || T(a.dt) * nu1[n] > T(1)) big = true;
+                        if (big && a.out_mode == OUT_EULER) fin_flags(a)[c] = 1;
                         store_row<T, N>(pnu + ((int64_t)rank * rows + r0) * N, nu0);
                         store_row<T, N>(pnu + ((int64_t)rank * rows + r1) * N, nu1);
                         continue;

@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
         if (S > 1) {
             pnu = reinterpret_cast<T *>(a.part) + (c * (S + 1) + S) * CELL;
             pg = reinterpret_cast<T *>(a.part) + (c * (S + 1) + prt) * CELL;
+            if (rank == 0 && tid == 0 && (a.paired ? o0 == 0 : o1 == a.nops)) fin_flags(a)[c] = 0;
         }
         const int64_t coff = a.cell_off ? a.cell_off[c] : c * CELL;
         const int64_t cglob = a.cell_id ? a.cell_id[c] : c;
@@ -449,7 +450,12 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
 #pragma unroll
                             for (int n = 0; n < M; ++n) nu[n] = half ? z[n].y : z[n].x;
                             if (S > 1) {
+                                bool over = false;
+#pragma unroll
+                                for (int n = 0; n < M; ++n)
+                                    if (a.dt * nu[n] > 1.0) over = true;
                                 if (has) quad_store<M>(pnu + grow * N + xb, nu);
+                                if (has && over && a.out_mode == OUT_EULER) fin_flags(a)[c] = 1;
                                 continue;
                             }
                             quad_load<M>(F + grow * N + xb, fr);

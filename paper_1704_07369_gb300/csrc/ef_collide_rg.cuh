@@ -398,7 +398,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
         const int64_t c = S > 1 ? w / S : w;
         const int prt = S > 1 ? (int)(w - c * S) : 0;
         int o0 = 0, o1 = a.nops;
-        if (SPLIT) split_range(a, prt, o0, o1);
+        if constexpr (SPLIT) {
+            split_range(a, prt, o0, o1);
+            if (o0 == 0 && rank == 0 && tid == 0) fin_flags(a)[c] = 0;      // (the loss comes first)
+        }
         const int64_t coff = a.cell_off ? a.cell_off[c] : c * CELL;
         const int64_t cglob = a.cell_id ? a.cell_id[c] : c;
         const T *F = reinterpret_cast<const T *>(a.F) + coff;
@@ -476,6 +479,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
         for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
             const bool pair = op.kind >= OP_PAIR;
+            bool told = false;             // (warp-uniform) this warp has flagged the cell
             // ---------------- A: multiply, axis 0 inverse, scatter (one (direction, pencil) item
             // per thread; lanes of a pair share the direction since NPC is even)
             const int nitems = (pair ? 2 : 1) * NPC;
@@ -615,7 +619,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                             T fr[N];
                             if (S > 1) {
 #pragma unroll
-                                for (int n = 0; n < N; ++n) fr[n] = j ? z[n].y : z[n].x;
+                                for (int n = 0; n < N; ++n) {
+                                    fr[n] = j ? z[n].y : z[n].x;
+                                    if (T(a.dt) * fr[n] > T(1)) bigt = true;
+                                }
                                 store_row<T, N>(pnu + ((int64_t)rank * rows + r) * N, fr);
                                 continue;
                             }
@@ -653,7 +660,10 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         T fr[N];
                         if (S > 1) {
 #pragma unroll
-                            for (int n = 0; n < N; ++n) fr[n] = z[n].x;
+                            for (int n = 0; n < N; ++n) {
+                                fr[n] = z[n].x;
+                                if (T(a.dt) * fr[n] > T(1)) bigt = true;
+                            }
                             store_row<T, N>(pnu + ((int64_t)rank * rows + r) * N, fr);
                             continue;
                         }
@@ -669,7 +679,11 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         mxt = mx > mxt ? mx : mxt;
                     }
                 }
-                if (bigt && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
+                if (bigt && a.out_mode == OUT_EULER) {
+                    if (S > 1) fin_flags(a)[c] = 1;
+                    else flag_cluster(cl, C, s_nubig);
+                }
+                told = ASYNC && S == 1 && __any_sync(wmask, bigt);
 #pragma unroll
                 for (int o2 = 16; o2 > 0; o2 >>= 1) {
                     const T u = __shfl_xor_sync(wmask, mxt, o2);
@@ -678,8 +692,8 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                 if (lane == 0) s_maxnu[tid >> 5] = mxt;
             }
             // write-after-read: the next op's scatter waits for this arrival.  With st.async no other
-            // barrier orders the loss op's flag of the cell, so that arrival releases it
-            if (ASYNC && !pair) bar.release_arrive();
+            // barrier orders what flag_cluster has written, so the warps that wrote release it here
+            if (told) bar.release_arrive();
             else bar.war_arrive();
             if (o + 1 == o1) {
                 bar.war_wait();

@@ -63,7 +63,8 @@ struct CollideArgs {
     void *part = nullptr;     // nsplit > 1: [cell][nsplit + 1][N^d] gain of each part, then nu; summed and
                               // written out by the finishing kernel (ef_split.cu)
     int fin_ctas = 1;         // its CTAs per cell, and their meeting place: arrivals [cell], zero between
-    void *fin = nullptr;      // launches; fin_off bytes on, the CTAs' diagnostics [cell][fin_ctas][kDiag]
+    void *fin = nullptr;      // launches; fin_off / 2 bytes on, flags [cell] that the collide launch leaves;
+                              // fin_off bytes on, the CTAs' diagnostics [cell][fin_ctas][kDiag]
     size_t fin_off = 0;
     long long slab_ns = 1000000000;   // limit of a wait for a slab's bytes (ef_collide_rg.cuh)
     int slab_extra = 0;       // bytes a slab expects and nobody sends: lets such waits run out (tests)

@@ -646,8 +646,9 @@ void cache_store(const std::string &key, int C, int tpb, int sg, int pf, int pr,
     std::fclose(f);
 }
 
-// arrivals of n cells, and the diagnostics of the CTAs of at most n (split_finish_ctas)
-size_t fin_offset(int64_t n) { return ((size_t)n * sizeof(int) + 255) / 256 * 256; }
+// arrivals and flags of n cells (the first and second half), and the diagnostics of the CTAs of at most n
+// (split_finish_ctas)
+size_t fin_offset(int64_t n) { return 2 * (((size_t)n * sizeof(int) + 255) / 256 * 256); }
 size_t fin_diag_bytes(int64_t n, int sms) { return ((size_t)std::max<int64_t>(n, 4 * (int64_t)sms) * ef::kDiag * 8 + 255) / 256 * 256; }
 
 // Plan-time autotuner: time every candidate shape (and the L1 prefetch on / off), as an Euler step

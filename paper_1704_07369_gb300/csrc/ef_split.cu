@@ -29,7 +29,6 @@ namespace ef {
 namespace {
 
 constexpr int kFinThreads = 128;     // one warp per sub-partition
-constexpr int kFinMax = 1023;        // CTAs per cell
 
 // values per thread and pass (split_finish_ctas has them too): 2D FP64 cells are small, so one
 template <typename T, int D>
@@ -89,7 +88,11 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
 
     DG dg;
     dg.reset();
-    bool bad = false, neg = false, big = false;      // an updated value below zero, dt nu > 1
+    bool bad = false, neg = false;           // an updated value below zero
+    // dt nu > 1 somewhere in the cell: the part with the loss has left it (ef_collide_impl.cuh, fin_flags).
+    // Loaded here, beside F, and not where it is used: its latency would end the launch
+    unsigned big;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(big) : "l"(fin_flags(a) + c));
     if (ROWS && a.diag) {
         // FP32: the sums over F by rows, in the order of emit_row, so that a cell's moments do not
         // depend on whether its launch was split
@@ -142,7 +145,6 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
             if (a.out_mode == OUT_EULER) {
                 o = f[j] + T(a.dt) * qv;
                 if (o < T(0)) neg = true;
-                if (T(a.dt) * nu[j] > T(1)) big = true;
             }
             if (!isfinite(o)) bad = true;
             if (a.diag) {
@@ -178,14 +180,8 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
         }
     }
     if (bad) record_status(a.status, 7);     // EF_ERR_NOT_FINITE
-    const bool euler = a.out_mode == OUT_EULER;
-    if (!euler && !a.diag) return;
-    // positivity is a property of the whole cell (ef_collide_impl.cuh, flag_cluster)
-    bool any_neg = false, any_big = false;
-    if (euler) {
-        any_neg = __syncthreads_or(neg);
-        any_big = __syncthreads_or(big);
-    }
+    if (a.out_mode == OUT_EULER && neg && big) record_status(a.status, 6);     // EF_ERR_POSITIVITY
+    if (!a.diag) return;
 
     auto merge = [](int k, double v, double u) { return (k == 7 || k == 9) ? fmin(v, u) : (k == 8 ? fmax(v, u) : v + u); };
     auto extreme = [](int k, auto x) {
@@ -196,9 +192,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
         }
         return x;
     };
-    if (!a.diag) {
-        // only the flags meet
-    } else if constexpr (FFD) {
+    if constexpr (FFD) {
 #pragma unroll
         for (int k = 0; k < 7; ++k) {
             FF x = dg.sum[k];
@@ -215,7 +209,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
         const double t = warp_sum8(v, lane);
         if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
     }
-    if (a.diag) {
+    {
         const double mf = extreme(7, dg.min_f), mx = extreme(8, dg.max_nu), mo = extreme(9, dg.min_out);
         if (lane == 0) {
             red[warp][7] = mf;
@@ -233,33 +227,24 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const CollideArgs a
         a.diag[cglob * kDiag + k] = v;
     };
     double *cta = reinterpret_cast<double *>(static_cast<unsigned char *>(a.fin) + a.fin_off) + c * C * kDiag;   // [C][kDiag]
-    if (a.diag && tid < kDiag) {
+    if (tid < kDiag) {
         double v = red[0][tid];
         for (int w = 1; w < kFinThreads / 32; ++w) v = merge(tid, v, red[w][tid]);
         if (C == 1) finish(tid, v);
         else cta[rank * kDiag + tid] = v;
     }
-    if (C == 1) {
-        if (tid == 0 && any_neg && any_big) record_status(a.status, 6);     // EF_ERR_POSITIVITY
-        return;
-    }
-    // the CTA that arrives last sums the cell's CTAs in order, and leaves the count at zero: arrivals in
-    // bits 0 - 9, CTAs with a value below zero in 10 - 19, CTAs with dt nu > 1 in 20 - 29 (C <= kFinMax)
+    if (C == 1) return;
+    // the CTA that arrives last sums the cell's CTAs in order, and leaves the arrival count at zero
     __shared__ int last;
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        unsigned *count = static_cast<unsigned *>(a.fin) + c;
-        const unsigned mine = 1u | (any_neg ? 1u << 10 : 0u) | (any_big ? 1u << 20 : 0u);
-        const unsigned all = atomicAdd(count, mine) + mine;
-        last = (all & 1023u) == (unsigned)C;
-        if (last) {
-            *count = 0;
-            if ((all >> 10 & 1023u) && all >> 20) record_status(a.status, 6);
-        }
+        int *count = static_cast<int *>(a.fin) + c;
+        last = atomicAdd(count, 1) == C - 1;
+        if (last) *count = 0;
     }
     __syncthreads();
-    if (!last || !a.diag) return;
+    if (!last) return;
     __threadfence();
     if (C <= 8) {
         if (tid < kDiag) {
@@ -300,7 +285,7 @@ cudaError_t finish_td(int N, const CollideArgs &a, cudaStream_t s)
 int split_finish_ctas(int prec, int d, int N, int64_t n, int sms)
 {
     const int W = prec == 0 ? 4 : d == 3 ? 2 : 1, rows = d == 3 ? N * N : N;
-    const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kFinMax, (int64_t)4 * sms / std::max<int64_t>(n, 1)));
+    const int64_t most = std::max<int64_t>(1, (int64_t)4 * sms / std::max<int64_t>(n, 1));
     const int rpc = (int)std::max<int64_t>((kFinThreads * W + N - 1) / N, (rows + most - 1) / most);
     return (rows + rpc - 1) / rpc;
 }
