@@ -298,14 +298,6 @@ __device__ __forceinline__ void store_row(T *dst, const T (&x)[N])
 // Positivity: an Euler step sets EF_ERR_POSITIVITY where a cell has an updated value below zero and
 // dt nu > 1 somewhere (dt max nu <= 1 keeps F >= 0, so there a value below zero is rounding).  Both are
 // properties of the whole cell, so that the report does not depend on how the cell is spread over CTAs.
-// Paired op lists know nu first: a CTA that sees dt nu > 1 tells every CTA of the cluster (flag is the
-// same variable of each), which read it in the last op, behind a release / acquire barrier.
-__device__ __forceinline__ void flag_cluster(cg::cluster_group &cl, int C, int *flag)
-{
-    if (atomicExch(flag, 1) == 0)
-        for (int r = 0; r < C; ++r) *cl.map_shared_rank(flag, r) = 1;
-}
-
 // A split launch's flag of each cell, dt nu > 1 somewhere in it: cleared and set by the part that holds the
 // loss, read by the finishing kernel (ef_split.cu).  (Findings that met in the finishing kernel itself cost a
 // small step 2 us of 12 - 19, for barriers or the latency of an atomic.)
@@ -378,6 +370,15 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, int rank)
     uint32_t r;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
+}
+// Paired op lists know nu first: whoever sees dt nu > 1 tells every CTA of the cluster (flag is the same
+// variable of each), which read it in the last op, behind a release / acquire barrier.  A warp's existing lanes
+// (wmask) share the stores, or a thread alone makes them (lane 0, mask 1).  No atomic decides who does: with it
+// the register kernels, which hold G here, spilled up to 130 bytes a thread more.
+__device__ __forceinline__ void flag_cluster(int *flag, int C, int lane, unsigned wmask)
+{
+    for (int r = lane; r < C; r += __popc(wmask))
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32addr(flag), r)), "r"(1) : "memory");
 }
 __device__ __forceinline__ void st_cluster(uint32_t a, float4 v)
 {
@@ -670,7 +671,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OC
         Diag dg;
         dg.reset();
         bool have_g = false;                // split: this part's G is already set
-        unsigned found = 0;                 // single-slab Euler step: what this thread's rows show (meet_positivity)
+        unsigned found = 0;                 // Euler step: what this thread's rows show (meet_positivity, flag_cluster)
 
         for (int o = o0; o < o1; ++o) {
             const Op op = a.ops[o];
@@ -809,7 +810,7 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OC
                             }
                             dg.max_nu = fmax(dg.max_nu, (double)mx);
                         }
-                        if (big && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
+                        if (big) found |= 2;
                     } break;
                     default: {  // OP_LOSS (single mode, last): Q = G - F nu; output; diagnostics
 #pragma unroll
@@ -835,6 +836,9 @@ __global__ void __launch_bounds__(OCC == 1 ? max_threads<N>() : kOcc2Threads, OC
                     } break;
                     }
                 }
+                // paired: the cell's dt nu > 1 to the cluster
+                if (op.kind == OP_NU_INIT && S == 1 && a.out_mode == OUT_EULER && __any_sync(0xffffffffu, found))
+                    flag_cluster(s_nubig, C, lane, 0xffffffffu);
                 if (op.kind == OP_G_SET || op.kind == OP_G_ADD) have_g = true;
             }
             bar.war();

@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) collide_kernel_q(const Collid
                                 if (has) {
 #pragma unroll
                                     for (int n = 0; n < M; ++n) Gr[n * rows] = -fr[n] * nu[n];
-                                    if (big && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
+                                    if (big && a.out_mode == OUT_EULER) flag_cluster(s_nubig, C, 0, 1u);
                                 }
                             } else {
 #pragma unroll

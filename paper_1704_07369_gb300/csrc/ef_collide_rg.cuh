@@ -679,11 +679,14 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
                         mxt = mx > mxt ? mx : mxt;
                     }
                 }
-                if (bigt && a.out_mode == OUT_EULER) {
-                    if (S > 1) fin_flags(a)[c] = 1;
-                    else flag_cluster(cl, C, s_nubig);
+                if (a.out_mode == OUT_EULER) {
+                    if constexpr (SPLIT) {
+                        if (bigt) fin_flags(a)[c] = 1;
+                    } else {
+                        told = __any_sync(wmask, bigt);
+                        if (told) flag_cluster(s_nubig, C, lane, wmask);
+                    }
                 }
-                told = ASYNC && S == 1 && __any_sync(wmask, bigt);
 #pragma unroll
                 for (int o2 = 16; o2 > 0; o2 >>= 1) {
                     const T u = __shfl_xor_sync(wmask, mxt, o2);
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(LB, 1) collide_kernel_rg(const CollideArgs a)
             }
             // write-after-read: the next op's scatter waits for this arrival.  With st.async no other
             // barrier orders what flag_cluster has written, so the warps that wrote release it here
-            if (told) bar.release_arrive();
+            if (ASYNC && told) bar.release_arrive();
             else bar.war_arrive();
             if (o + 1 == o1) {
                 bar.war_wait();

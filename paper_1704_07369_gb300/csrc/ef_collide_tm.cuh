@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(LB, MINB) collide_kernel_tm(const CollideArgs 
                     }
                     mxt = mx > mxt ? mx : mxt;
                 }
-                if (bigt && a.out_mode == OUT_EULER) flag_cluster(cl, C, s_nubig);
+                if (a.out_mode == OUT_EULER && __any_sync(wmask, bigt)) flag_cluster(s_nubig, C, lane, wmask);
 #pragma unroll
                 for (int o2 = 16; o2 > 0; o2 >>= 1) {
                     const T u = __shfl_xor_sync(wmask, mxt, o2);
