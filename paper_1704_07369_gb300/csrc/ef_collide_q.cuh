@@ -18,8 +18,8 @@
 // it then holds the outputs k + (N/4) t(s), k < N/4, t the bit reversal of s: a contiguous block.
 //
 // Measured against one thread per line with N/2 + 1 columns (both split alike, with the first finishing kernel): Q of 24
-// cells of N = 64 13.3 -> 10.4 ms (of which the FP64 pipe needs 5.8 ms on all SMs, 6.9 on the 128 that
-// clusters of 16 reach), two Euler steps of one cell of N = 32 1.11 -> 0.925 ms, 100 steps of one 2D
+// cells of N = 64 13.3 -> 10.4 ms (of which the FP64 pipe needs 5.8 ms on all SMs, 7.9 on the 112 that the
+// 7 resident clusters of 16 reach), two Euler steps of one cell of N = 32 1.11 -> 0.925 ms, 100 steps of one 2D
 // cell of N = 16 4.7 -> 2.87 ms, two SSP-RK3 steps of four 2D cells of N = 64 1.17 -> 0.87 ms.
 #pragma once
 
